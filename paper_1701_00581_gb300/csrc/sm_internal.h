@@ -29,6 +29,9 @@ static_assert(TILE_V == 32, "a tile row of offsets maps onto the 32 lanes of a w
 constexpr int REF_W = TILE_W, REF_U = (WBY + VBY - 1) * (WBX + VBX - 1), REF_V = TILE_V;
 constexpr int REF_SLOTS = REF_W + REF_U + REF_V;   // 413
 
+// Batches of the phase recursion (k_phase.cu): points and late terms at most.
+constexpr int PHASE_BATCH_MIN = 64, PHASE_BATCH_MAX = 128, PHASE_LATE = 768;
+
 constexpr float FP16_SCALE = 16384.0f;       // |I_n| <= 1 -> fits half with margin
 constexpr float FP16_INV_SCALE = 1.0f / 16384.0f;
 
@@ -65,13 +68,19 @@ struct PlanDev {
     const int* wb_tiles;
     // phase recursion work items: (point, tile) pairs holding at least one
     // pair the point reads, grouped by point, points in ring order
-    const int4* items;          // [n_items] packed (w, offset origin) bytes, B offset
-                                //   within the subfield, mask of lanes whose pair is read
-    const int* ring_items;      // [n_rings + 1] first item of each ring
-    const int* point_items;     // [n_points + 1] first item of each point
-    const int4* point_rec;      // [n_points] (wx, wy, first item, end item), items counted
-                                //   from the first item of the point's ring
-    int n_items, max_ring_items, max_ring_points;
+    // phase recursion (k_phase.cu): batches of rings; per point the tile rows
+    // holding its early terms and the list of its late ones; a frequency's
+    // signed index is (ky * zpitch + kx) * bytes of a phasor
+    const int2* items;          // (tile * TILE_W * VBY + row, signed index of the row's first offset << 8 |
+                                //   mask of the row's early offsets), by point in ring order
+    const int2* late;           // late terms (B offset within the subfield, signed index of v), by point
+    const int2* units;          // early units: (first of items, up to 32 items | point within its batch << 6)
+    const int4* point_rec;      // [n_points + 1] (signed index of w, first of units, first of late,
+                                //   target slot in its tiles)
+    const int* batch_ring;      // [n_batches + 1] first ring of each batch
+    const int* batch_unit;      // [n_batches + 1] first unit of each batch
+    int n_batches, max_batch_points, max_batch_units, max_batch_late;
+    int zpitch;                 // row pitch of the recursion's phasor table and of its signed indices
     // seeing (Sect. 3.1): the non-overlapping N x N cubes among the
     // subfields and the annuli of unit width over the half-plane domain
     int n_cubes;
@@ -156,6 +165,5 @@ int batch_blocks_per_sm(size_t smem, int prec, int minb);
 cudaError_t launch_batch(const smi::BatchArgs& a, int prec, int minb, const int4* items, int n_items, int* head,
                          int* cnt, int* status, float2* scratch, size_t scr_elems, int grid, size_t smem,
                          cudaStream_t st);
-size_t phase_smem_bytes(int hb_rows, int box_pitch, int max_ring_items, int max_ring_points,
-                        int phase_prec);
+size_t phase_smem_bytes(int hb_rows, int zpitch, int max_points, int max_units, int max_late, int phase_prec);
 }  // namespace smk

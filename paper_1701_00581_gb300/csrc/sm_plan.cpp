@@ -94,7 +94,7 @@ int validate_channel(const sm_channel* ch) {
         set_error("fc*N too large for the shared-memory FFT at this N"); return SM_EINVAL;
     }
     const int pitch = ((2 * K + 1) + 3) / 4 * 4;
-    if (smk::phase_smem_bytes(K + 1, pitch, 0, 0, ch->phase_prec) > 200 * 1024) {
+    if ((size_t)(K + 1) * pitch * (ch->phase_prec == SM_PHASE_FP32 ? 8 : 16) > 200 * 1024) {
         set_error("phase table exceeds shared memory"); return SM_EINVAL;
     }
     return SM_OK;
@@ -309,46 +309,128 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.n_points = (int)pts.size();
     d.n_rings = (int)pl->ring_start.size() - 1;
 
-    // recursion work items: for each point (ring order), the tiles of its
-    // w-block that hold at least one pair the point reads
-    pl->point_items.assign(d.n_points + 1, 0);
-    pl->items.clear();
-    for (int pi = 0; pi < d.n_points; ++pi) {
-        const int wx = pts[pi].x, wy = pts[pi].y;
-        const int wb = (wy / WBY) * d.n_wbx + (wx + K) / WBX;
-        pl->point_items[pi] = (int)pl->items.size();
-        for (int ti = pl->wb_start[wb]; ti < pl->wb_start[wb + 1]; ++ti) {
-            const int t = pl->wb_tiles[ti];
-            const int4 T = pl->tiles[t];
-            unsigned mask = 0;
-            for (int l = 0; l < TILE_V; ++l)
-                if (pair_used_host(wx, wy, T.z + l % VBX, T.w + l / VBX, r2i, R * R)) mask |= 1u << l;
-            if (!mask) continue;
-            const unsigned packed = (unsigned)(wx & 255) | ((unsigned)(wy & 255) << 8) |
-                                    ((unsigned)(T.z & 255) << 16) | ((unsigned)(T.w & 255) << 24);
-            const int wxl = (wx + K) % WBX, wyl = wy % WBY;
-            const int boff = t * TILE_PAIRS + (wyl * WBX + wxl) * TILE_V;
-            pl->items.push_back(make_int4((int)packed, boff, (int)mask, 0));
+    // Phase recursion (k_phase.cu).  Batches of consecutive rings, at most
+    // PHASE_BATCH points and PHASE_LATE late terms each (a ring by itself has
+    // none).  Per point the late terms -- u or v on an earlier ring of the
+    // point's own batch -- in order of v, and the tile rows of its w-block
+    // that hold an early one.
+    //
+    // The phasor table's pitch is 8 (mod 16) complex floats, so that the two
+    // rows of offsets that half a warp reads fall on different banks; wider
+    // values, or a table that would not fit, take the box's own pitch.
+    int per_batch = std::max(PHASE_BATCH_MIN, std::min(PHASE_BATCH_MAX, d.n_points / 32));
+    d.zpitch = d.box_pitch;
+    if (d.phase_prec == SM_PHASE_FP32) {
+        const int padded = (2 * K + 2 + 7) / 16 * 16 + 8;
+        const int most_units = per_batch * (nvb * VBY / 32 + 1);
+        if (smk::phase_smem_bytes(d.hb_rows, padded, per_batch, most_units, PHASE_LATE, d.phase_prec) <= 227 * 1024)
+            d.zpitch = padded;
+    }
+    const int zb = d.phase_prec == SM_PHASE_FP32 ? 8 : 16;     // bytes of a phasor
+    int max_ring_entries = 0, max_ring_points = 0;
+    for (;; per_batch /= 2) {
+        pl->batch_ring.assign(1, 0);
+        pl->batch_unit.assign(1, 0);
+        pl->items.clear();
+        pl->units.clear();
+        pl->late.clear();
+        pl->point_rec.resize(d.n_points + 1);
+        d.max_batch_points = d.max_batch_units = d.max_batch_late = 0;
+        max_ring_entries = max_ring_points = 0;
+        {
+            std::vector<int> entry(d.n_tiles, -1);           // the point's first list entry of a tile
+            std::vector<std::vector<int2>> ring_late;        // the ring's points' late offsets v
+            auto before = [](const int2& a, const int2& b) { return a.y != b.y ? a.y < b.y : a.x < b.x; };
+            auto same = [](const int2& a, const int2& b) { return a.x == b.x && a.y == b.y; };
+            size_t batch_late = 0;
+            for (int rr = 0; rr < d.n_rings; ++rr) {
+                const int p0 = pl->ring_start[rr], p1 = pl->ring_start[rr + 1];
+                int first = pl->ring_start[pl->batch_ring.back()];
+                ring_late.assign(p1 - p0, {});
+                size_t nlate = 0;
+                for (int pi = p0; pi < p1; ++pi) {
+                    const int wx = pts[pi].x, wy = pts[pi].y;
+                    std::vector<int2>& vs = ring_late[pi - p0];
+                    for (int pj = first; pj < p0; ++pj)
+                        for (int sg = -1; sg <= 1; sg += 2) {
+                            const int x = sg * pts[pj].x, y = sg * pts[pj].y;
+                            if (pair_used_host(wx, wy, wx - x, wy - y, r2i, R * R)) vs.push_back(make_int2(wx - x, wy - y));
+                            if (pair_used_host(wx, wy, x, y, r2i, R * R)) vs.push_back(make_int2(x, y));
+                        }
+                    std::sort(vs.begin(), vs.end(), before);
+                    vs.erase(std::unique(vs.begin(), vs.end(), same), vs.end());
+                    nlate += vs.size();
+                }
+                if (p1 - first > per_batch || batch_late + nlate > (size_t)PHASE_LATE) {      // a new batch starts here
+                    if (p0 > first) {
+                        pl->batch_ring.push_back(rr);
+                        pl->batch_unit.push_back((int)pl->units.size());
+                        first = p0;
+                        batch_late = nlate = 0;
+                        ring_late.assign(p1 - p0, {});
+                    }
+                }
+                batch_late += nlate;
+                d.max_batch_late = std::max(d.max_batch_late, (int)batch_late);
+                d.max_batch_points = std::max(d.max_batch_points, p1 - first);
+                max_ring_points = std::max(max_ring_points, p1 - p0);
+                int ring_entries = 0;
+                for (int pi = p0; pi < p1; ++pi) {
+                    const int wx = pts[pi].x, wy = pts[pi].y;
+                    const int wb = (wy / WBY) * d.n_wbx + (wx + K) / WBX;
+                    const int slot = (wy % WBY) * WBX + (wx + K) % WBX;
+                    pl->point_rec[pi] = make_int4((wy * d.zpitch + wx) * zb, (int)pl->units.size(), (int)pl->late.size(), slot);
+                    const size_t e0 = pl->items.size();
+                    for (int ti = pl->wb_start[wb]; ti < pl->wb_start[wb + 1]; ++ti) {
+                        const int t = pl->wb_tiles[ti];
+                        const int4 T = pl->tiles[t];
+                        unsigned mask = 0;
+                        for (int l = 0; l < TILE_V; ++l)
+                            if (pair_used_host(wx, wy, T.z + l % VBX, T.w + l / VBX, r2i, R * R)) mask |= 1u << l;
+                        if (!mask) continue;
+                        ++ring_entries;
+                        entry[t] = (int)pl->items.size();
+                        for (int c = 0; c < VBY; ++c) {
+                            const int iv = ((T.w + c) * d.zpitch + T.z) * zb;
+                            pl->items.push_back(make_int2(t * TILE_W * VBY + c,
+                                                          (int)((unsigned)iv << 8 | (mask >> (VBX * c) & 0xffu))));
+                        }
+                    }
+                    for (const int2& v : ring_late[pi - p0]) {
+                        const int vbx = (v.x - d.v_org) / VBX, vby = (v.y + R) / VBY;
+                        const int t = pl->tile_of[(size_t)wb * nvb + vby * pl->n_vbx + vbx];
+                        const int l = (v.y + R - vby * VBY) * VBX + (v.x - d.v_org - vbx * VBX);
+                        pl->items[entry[t] + l / VBX].y &= ~(1 << l % VBX);
+                        pl->late.push_back(make_int2(t * TILE_PAIRS + slot * TILE_V + l, (v.y * d.zpitch + v.x) * zb));
+                    }
+                    // drop the entries left without an early term
+                    pl->items.erase(std::remove_if(pl->items.begin() + e0, pl->items.end(),
+                                                   [](const int2& e) { return (e.y & 0xff) == 0; }), pl->items.end());
+                    for (size_t e = e0; e < pl->items.size(); e += 32)
+                        pl->units.push_back(make_int2((int)e, (int)std::min<size_t>(32, pl->items.size() - e) | (pi - first) << 6));
+                }
+                d.max_batch_units = std::max(d.max_batch_units, (int)pl->units.size() - pl->batch_unit.back());
+                max_ring_entries = std::max(max_ring_entries, ring_entries);
+            }
+            pl->batch_ring.push_back(d.n_rings);
+            pl->batch_unit.push_back((int)pl->units.size());
+            pl->point_rec[d.n_points] = make_int4(0, (int)pl->units.size(), (int)pl->late.size(), 0);
         }
+        d.n_batches = (int)pl->batch_ring.size() - 1;
+        // smaller batches where the sums of their units do not fit
+        if (per_batch <= 8 || smk::phase_smem_bytes(d.hb_rows, d.zpitch, d.max_batch_points, d.max_batch_units,
+                                                    d.max_batch_late, d.phase_prec) <= 227 * 1024)
+            break;
     }
-    pl->point_items[d.n_points] = (int)pl->items.size();
-    pl->ring_items.resize(d.n_rings + 1);
-    d.max_ring_items = 0;
-    for (int rr = 0; rr <= d.n_rings; ++rr) {
-        pl->ring_items[rr] = pl->point_items[pl->ring_start[rr]];
-        if (rr > 0) d.max_ring_items = std::max(d.max_ring_items, pl->ring_items[rr] - pl->ring_items[rr - 1]);
-    }
-    d.n_items = (int)pl->items.size();
-    d.max_ring_points = 0;
-    pl->point_rec.resize(d.n_points);
-    for (int rr = 0; rr < d.n_rings; ++rr) {
-        d.max_ring_points = std::max(d.max_ring_points, pl->ring_start[rr + 1] - pl->ring_start[rr]);
-        for (int pi = pl->ring_start[rr]; pi < pl->ring_start[rr + 1]; ++pi)
-            pl->point_rec[pi] = make_int4(pts[pi].x, pts[pi].y, pl->point_items[pi] - pl->ring_items[rr],
-                                          pl->point_items[pi + 1] - pl->ring_items[rr]);
-    }
-    if (smk::phase_smem_bytes(d.hb_rows, d.box_pitch, d.max_ring_items, d.max_ring_points, d.phase_prec) >
-        227 * 1024) {
+    // Limit of the recursion's tables: a ring's (point, tile) entries and the
+    // phasors have to fit 227 KB (the bound on R at a given fc N).
+    const size_t e2 = d.phase_prec == SM_PHASE_FP32 ? 8 : 16;
+    auto up16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    const size_t tables = up16((size_t)max_ring_entries * e2) + up16((size_t)d.hb_rows * d.box_pitch * e2) +
+                          (size_t)max_ring_entries * 16 + (size_t)max_ring_points * 32;
+    if (tables > 227 * 1024 || d.n_tiles > 0xffff ||
+        smk::phase_smem_bytes(d.hb_rows, d.zpitch, d.max_batch_points, d.max_batch_units, d.max_batch_late,
+                              d.phase_prec) > 227 * 1024) {
         delete pl;
         set_error("phase recursion tables exceed shared memory");
         return SM_EINVAL;
@@ -417,9 +499,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {pl->wb_start.data(), pl->wb_start.size() * sizeof(int), 0},
         {pl->wb_tiles.data(), pl->wb_tiles.size() * sizeof(int), 0},
         {t0.data(), t0.size() * sizeof(double), 0},
-        {pl->items.data(), pl->items.size() * sizeof(int4), 0},
-        {pl->ring_items.data(), pl->ring_items.size() * sizeof(int), 0},
-        {pl->point_items.data(), pl->point_items.size() * sizeof(int), 0},
+        {pl->items.data(), pl->items.size() * sizeof(int2), 0},
+        {pl->late.data(), pl->late.size() * sizeof(int2), 0},
+        {pl->batch_ring.data(), pl->batch_ring.size() * sizeof(int), 0},
         {winft.data(), winft.size() * sizeof(float2), 0},
         {pl->point_rec.data(), pl->point_rec.size() * sizeof(int4), 0},
         {pl->cube_of_sub.data(), pl->cube_of_sub.size() * sizeof(int), 0},
@@ -428,6 +510,8 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {pl->ref_start.data(), pl->ref_start.size() * sizeof(int), 0},
         {pl->ref_idx.data(), pl->ref_idx.size() * sizeof(int), 0},
         {pl->tile_masks.data(), pl->tile_masks.size() * sizeof(unsigned), 0},
+        {pl->units.data(), pl->units.size() * sizeof(int2), 0},
+        {pl->batch_unit.data(), pl->batch_unit.size() * sizeof(int), 0},
     };
     size_t total = 0;
     for (auto& p : pcs) { p.off = total; total += align256(std::max<size_t>(p.bytes, 1)); }
@@ -452,9 +536,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.wb_start = (const int*)at(8);
     d.wb_tiles = (const int*)at(9);
     d.t0 = (const double*)at(10);
-    d.items = (const int4*)at(11);
-    d.ring_items = (const int*)at(12);
-    d.point_items = (const int*)at(13);
+    d.items = (const int2*)at(11);
+    d.late = (const int2*)at(12);
+    d.batch_ring = (const int*)at(13);
     d.winft = (const float2*)at(14);
     d.point_rec = (const int4*)at(15);
     d.cube_of_sub = (const int*)at(16);
@@ -463,6 +547,8 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.ref_start = (const int*)at(19);
     d.ref_idx = (const int*)at(20);
     d.tile_masks = (const unsigned*)at(21);
+    d.units = (const int2*)at(22);
+    d.batch_unit = (const int*)at(23);
     *out = pl;
     return SM_OK;
 }

@@ -18,9 +18,9 @@ struct sm_plan {
     std::vector<int> wb_start, wb_tiles;
     std::vector<int> ring_start;
     std::vector<int2> points;
-    std::vector<int4> items;
-    std::vector<int> ring_items, point_items;
+    std::vector<int2> items, units, late;   // phase recursion: early tile rows, units of them, late terms
     std::vector<int4> point_rec;
+    std::vector<int> batch_ring, batch_unit;
     std::vector<int> cubes, cube_of_sub;   // seeing cubes (subfield ids), subfield -> cube or -1
     std::vector<int> ann_start, ann_idx;   // annuli of the half-plane domain
     std::vector<int> ref_start, ref_idx;   // refinement partial slots of each recursion point
