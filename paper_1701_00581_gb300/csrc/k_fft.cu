@@ -5,51 +5,20 @@
 // the separable window, its windowed mean is removed, and the 2-D DFT is
 // taken as real row FFTs (two rows packed per complex FFT) followed by
 // column FFTs of only the K+1 non-negative columns inside the cutoff box.
-// The forward transforms are four-step FFTs (N = P x Q) computed in
-// registers by groups of 16 threads with one shared-memory exchange; the
-// inverse (one CTA per subfield, off the critical path) uses warp-wide
-// radix-2 Stockham FFTs in shared memory.
+// The transforms are four-step FFTs (N = P x Q) computed in registers by
+// groups of 16 threads with one shared-memory exchange.
 #include "sm_fft_dev.cuh"
 
 namespace {
 
 using smi::PlanDev;
-using smf::cmul;
 using smf::four_step;
 using smf::load_sample;
 using smf::Split;
 using smf::store_spec;
 
-// Radix-2 Stockham FFT of length N by one warp.  a holds the input, b is
-// scratch; returns the buffer holding the output in natural order.
-// INV = true uses exp(+2 pi i k / N) (unnormalised inverse).
-template <int N, bool INV>
-__device__ __forceinline__ float2* warp_fft(float2* a, float2* b, const float2* tw, int lane) {
-#pragma unroll
-    for (int Ns = 1; Ns < N; Ns <<= 1) {
-#pragma unroll
-        for (int j = lane; j < N / 2; j += 32) {
-            const int k = j & (Ns - 1);
-            float2 w = tw[k * (N / (2 * Ns))];
-            if (INV) w.y = -w.y;
-            const float2 a0 = a[j];
-            const float2 t = cmul(a[j + N / 2], w);
-            const int o = 2 * j - k;
-            b[o] = make_float2(a0.x + t.x, a0.y + t.y);
-            b[o + Ns] = make_float2(a0.x - t.x, a0.y - t.y);
-        }
-        __syncwarp();
-        float2* t = a;
-        a = b;
-        b = t;
-    }
-    return a;
-}
-
-constexpr int FFT_THREADS = 256;
-constexpr int FFT_WARPS = FFT_THREADS / 32;
-// Forward transforms: 32 groups of 16 threads for N >= 128 (one CTA per SM
-// fits in shared memory, so latency is hidden by warps within the CTA).
+// 32 groups of 16 threads for N >= 128 (one CTA per SM fits in shared memory,
+// so latency is hidden by warps within the CTA).
 template <int N> struct SpecThreads { static constexpr int T = N >= 128 ? 512 : 256; };
 
 // Thread groups of the four-step transform: G threads per transform.
@@ -60,12 +29,9 @@ template <int N> struct Grp {
     static constexpr int TB = (Q * (P + 1) > N ? Q * (P + 1) : N);   // exchange buffer
 };
 
-// scratch area (float2): per-warp ping-pong of the inverse, per-group
-// exchange tiles of the forward transform
+// scratch area (float2): the groups' exchange tiles
 template <int N>
-__host__ __device__ constexpr int scratch_elems() {
-    return FFT_WARPS * 2 * N > Grp<N>::NG * Grp<N>::TB ? FFT_WARPS * 2 * N : Grp<N>::NG * Grp<N>::TB;
-}
+__host__ __device__ constexpr int scratch_elems() { return Grp<N>::NG * Grp<N>::TB; }
 __host__ __device__ constexpr int scratch_elems_rt(int N) {
     return N == 64 ? scratch_elems<64>() : (N == 128 ? scratch_elems<128>() : scratch_elems<256>());
 }
@@ -76,7 +42,7 @@ __host__ __device__ constexpr size_t fft_smem(int N, int K) {
            + (size_t)N * sizeof(float2)                      // twiddles
            + (size_t)(K + 1) * sizeof(float2)                // window transform
            + (size_t)2 * N * sizeof(float)                   // windows
-           + (size_t)(FFT_WARPS * 2 + 2) * sizeof(double);   // reductions and scalars
+           + (size_t)18 * sizeof(double);                    // reductions and scalars
 }
 
 // Spectra of one (frame, subfield): the tile times the window is transformed
@@ -243,12 +209,30 @@ k_spectra(PlanDev p, const TIn* __restrict__ frames, int F, int sub0, void* __re
     }
 }
 
+// a * v rounded to FP32.  The FP32 recursion's phasors are FP64 copies of
+// floats: their bits are repacked on the integer pipe and multiplied in FP32,
+// which rounds the same exact product; anything else takes the FP64 product
+// (GB300's FP64 unit converts and multiplies two values per clock and SM).
+__device__ __forceinline__ float scaled(float a, double v) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int e = (hi >> 20) & 0x7ff;
+    if (e < 897 || e > 1150 || (lo & 0x1fffffff)) return (float)(a * v);
+    return a * __int_as_float((hi & 0x80000000) | ((e - 896) << 23) | ((hi & 0xfffff) << 3) | ((unsigned)lo >> 29));
+}
+
 // Inverse: O = A z on the disk (Hermitian), DC removed; columns first, then
-// pairs of Hermitian rows packed into one complex inverse FFT.
+// pairs of Hermitian rows packed into one complex inverse FFT, by the forward
+// transform's four-step groups.  304 subfields of
+// 256^2: 237 -> 85 us; 225 of 128^2: 66 -> 38 us; one of 64^2: 25 -> 12 us
+// (warp-wide radix-2 passes in shared memory, FP64 products and a serial sum
+// over the frames before).
 template <int N>
-__global__ void __launch_bounds__(FFT_THREADS, 1)
+__global__ void __launch_bounds__(SpecThreads<N>::T, 1)
 k_inverse(PlanDev p, int F, int sub0, const float* __restrict__ A, const double2* __restrict__ z,
           const float* __restrict__ flux, const float* __restrict__ mu, float* __restrict__ rec) {
+    using GP = Grp<N>;
+    constexpr int P = GP::P, Q = GP::Q, G = GP::G, NG = GP::NG, TB = GP::TB;
+    constexpr int TS = SpecThreads<N>::T, WS = TS / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, K1 = K + 1, CP = N + 1;
     float2* C = reinterpret_cast<float2*>(smem);
@@ -260,73 +244,89 @@ k_inverse(PlanDev p, int F, int sub0, const float* __restrict__ A, const double2
 
     const int sl = blockIdx.x, s = sub0 + sl;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int i = tid; i < N; i += FFT_THREADS) {
+    const int grp = tid / G, g = tid - grp * G;
+    float2* T = scratch + grp * TB;
+    for (int i = tid; i < N; i += TS) {
         stw[i] = p.tw[i];
         swx[i] = p.winx[(size_t)s * N + i];
         swy[i] = p.winy[(size_t)s * N + i];
     }
-    if (tid == 0) {
+    if (warp == 0) {
         double fs = 0.0, ms = 0.0;
-        for (int f = 0; f < F; ++f) {
+        for (int f = lane; f < F; f += 32) {
             fs += flux[(size_t)sl * F + f];
             ms += mu[(size_t)sl * F + f];
         }
-        red[0] = fs / F;
-        red[1] = ms / F;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            fs += __shfl_xor_sync(0xffffffffu, fs, o);
+            ms += __shfl_xor_sync(0xffffffffu, ms, o);
+        }
+        if (lane == 0) {
+            red[0] = fs / F;
+            red[1] = ms / F;
+        }
     }
+    for (int e = tid; e < K1 * CP; e += TS) C[e] = make_float2(0.f, 0.f);
+    __syncthreads();
+    // the half box row by row: (kx, ky) into column kx, its mirror (-kx, -ky)
+    // conjugated into column -kx
     const size_t hb = (size_t)p.hb_rows * p.box_pitch;
     const float* As = A + (size_t)sl * hb;
     const double2* zs = z + (size_t)sl * hb;
-    for (int e = tid; e < K1 * N; e += FFT_THREADS) {
-        const int kx = e / N, j = e - kx * N;
-        const int ky = j < N / 2 ? j : j - N;
-        float2 v = make_float2(0.f, 0.f);
-        if (kx * kx + ky * ky <= p.r2i && (kx | ky) != 0 && ky >= -K && ky <= K) {
-            if (ky > 0 || (ky == 0 && kx > 0)) {
-                const size_t o = (size_t)ky * p.box_pitch + kx + K;
-                const double2 zz = zs[o];
-                v = make_float2((float)(As[o] * zz.x), (float)(As[o] * zz.y));
-            } else {
-                const size_t o = (size_t)(-ky) * p.box_pitch + (-kx) + K;
-                const double2 zz = zs[o];
-                v = make_float2((float)(As[o] * zz.x), (float)(-As[o] * zz.y));
-            }
+    for (int ky = warp; ky <= K; ky += WS)
+        for (int col = lane; col < p.box_cols; col += 32) {
+            const int kx = col - K;
+            if (kx * kx + ky * ky > p.r2i || (ky == 0 && kx <= 0)) continue;
+            const size_t o = (size_t)ky * p.box_pitch + col;
+            const double2 zz = zs[o];
+            const float a = As[o];
+            const float2 v = make_float2(scaled(a, zz.x), scaled(a, zz.y));
+            if (kx >= 0) C[kx * CP + ky] = v;
+            if (kx <= 0) C[-kx * CP + N - ky] = make_float2(v.x, -v.y);
         }
-        C[kx * CP + j] = v;
-    }
     __syncthreads();
-    const double fmean = red[0];
     const float mmean = (float)red[1];
-    const float scale = (float)(fmean / ((double)N * N));
+    const float scale = (float)(red[0] / ((double)N * N));
 
-    float2* fa = scratch + warp * 2 * N;
-    float2* fb = fa + N;
-    for (int kx = warp; kx < K1; kx += FFT_WARPS) {
-        float2* col = C + (size_t)kx * CP;
-        for (int y = lane; y < N; y += 32) fa[y] = col[y];
-        __syncwarp();
-        const float2* Zc = warp_fft<N, true>(fa, fb, stw, lane);
-        for (int y = lane; y < N; y += 32) col[y] = Zc[y];
+    for (int c0 = 0; c0 < K1; c0 += NG) {
+        const int kx = c0 + grp;
+        const int kc = kx < K1 ? kx : K1 - 1;
+        float2 v[Q], X[P];
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) v[n2] = g < P ? C[kc * CP + g + P * n2] : make_float2(0.f, 0.f);
+        four_step<N, true>(v, X, T, stw, g);
+        if (kx < K1 && g < Q) {
+#pragma unroll
+            for (int k1 = 0; k1 < P; ++k1) C[kx * CP + g + Q * k1] = X[k1];
+        }
         __syncwarp();
     }
     __syncthreads();
 
     float* out = rec + (size_t)s * N * N;
-    for (int pr = warp; pr < N / 2; pr += FFT_WARPS) {
-        const int y1 = 2 * pr, y2 = y1 + 1;
-        for (int kx = lane; kx < N; kx += 32) fa[kx] = make_float2(0.f, 0.f);
+    for (int pr0 = 0; pr0 < N / 2; pr0 += NG) {
+        const int y1 = 2 * (pr0 + grp), y2 = y1 + 1;
+        for (int kx = g; kx < N; kx += G) T[kx] = make_float2(0.f, 0.f);
         __syncwarp();
-        for (int kx = lane; kx < K1; kx += 32) {
+        for (int kx = g; kx < K1; kx += G) {
             const float2 a = C[kx * CP + y1], b = C[kx * CP + y2];
-            fa[kx] = make_float2(a.x - b.y, a.y + b.x);
-            if (kx > 0) fa[N - kx] = make_float2(a.x + b.y, -a.y + b.x);
+            T[kx] = make_float2(a.x - b.y, a.y + b.x);
+            if (kx > 0) T[N - kx] = make_float2(a.x + b.y, -a.y + b.x);
         }
         __syncwarp();
-        const float2* Zr = warp_fft<N, true>(fa, fb, stw, lane);
-        for (int x = lane; x < N; x += 32) {
-            const float2 v = Zr[x];
-            out[(size_t)y1 * N + x] = v.x * scale + mmean * swx[x] * swy[y1];
-            out[(size_t)y2 * N + x] = v.y * scale + mmean * swx[x] * swy[y2];
+        float2 v[Q], X[P];
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) v[n2] = g < P ? T[g + P * n2] : make_float2(0.f, 0.f);
+        __syncwarp();
+        four_step<N, true>(v, X, T, stw, g);
+        if (g < Q) {
+#pragma unroll
+            for (int k1 = 0; k1 < P; ++k1) {
+                const int x = g + Q * k1;
+                out[(size_t)y1 * N + x] = X[k1].x * scale + mmean * swx[x] * swy[y1];
+                out[(size_t)y2 * N + x] = X[k1].y * scale + mmean * swx[x] * swy[y2];
+            }
         }
         __syncwarp();
     }
@@ -366,7 +366,7 @@ cudaError_t inverse_n(const PlanDev& p, int F, int sub0, int nsub, const float* 
     cudaError_t e = cudaFuncSetAttribute(k_inverse<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
     if (e != cudaSuccess) return e;
-    k_inverse<N><<<nsub, FFT_THREADS, sm, st>>>(p, F, sub0, A, z, flux, mu, rec);
+    k_inverse<N><<<nsub, SpecThreads<N>::T, sm, st>>>(p, F, sub0, A, z, flux, mu, rec);
     return cudaGetLastError();
 }
 

@@ -32,6 +32,10 @@ constexpr int REF_SLOTS = REF_W + REF_U + REF_V;   // 413
 // Batches of the phase recursion (k_phase.cu): points and late terms at most.
 constexpr int PHASE_BATCH_MIN = 64, PHASE_BATCH_MAX = 128, PHASE_LATE = 768;
 
+// D/r0 candidates of the seeing fit, log-spaced (k_seeing.cu).
+constexpr int SEEING_GRID = 256;
+constexpr double SEEING_LO = 1.0, SEEING_HI = 64.0;
+
 constexpr float FP16_SCALE = 16384.0f;       // |I_n| <= 1 -> fits half with margin
 constexpr float FP16_INV_SCALE = 1.0f / 16384.0f;
 
@@ -90,6 +94,9 @@ struct PlanDev {
     const int* ann_start;    // [n_bins + 1] CSR over ann_idx
     const int* ann_idx;      // half-box element index (ky * box_pitch + kx + K), row-major per annulus
     const double* t0;        // [hb_rows][box_pitch] diffraction OTF on the half box
+    const double* r53;       // [hb_rows][box_pitch] rho^(5/3), rho = |k| / rcut, on the half box
+    const double2* ann_model; // [n_bins] (T0, rho^(5/3)) at |k| = b, b < rcut
+    const double2* cand;     // [SEEING_GRID] (x^(5/3), ck / x^2) of the D/r0 candidates x
 };
 
 constexpr int MAX_BATCH = 8;

@@ -172,7 +172,7 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
 
     // diffraction OTF T0 on the half box
     const size_t hb = (size_t)d.hb_rows * d.box_pitch;
-    std::vector<double> t0(hb, 0.0);
+    std::vector<double> t0(hb, 0.0), r53(hb, 0.0);
     int nU = 0;
     for (int ky = -K; ky <= K; ++ky)
         for (int kx = -K; kx <= K; ++kx) {
@@ -181,6 +181,7 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
             ++nU;
             if (ky < 0) continue;
             const double rho = std::sqrt((double)q) / r;
+            r53[(size_t)ky * d.box_pitch + kx + K] = std::pow(rho, 5.0 / 3.0);
             t0[(size_t)ky * d.box_pitch + kx + K] =
                 rho <= 1.0 ? (2.0 / M_PI) * (std::acos(rho) - rho * std::sqrt(1.0 - rho * rho)) : 0.0;
         }
@@ -266,6 +267,18 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
             pl->ann_start[b + 1] = pl->ann_start[b] + (int)ann[b].size();
             pl->ann_idx.insert(pl->ann_idx.end(), ann[b].begin(), ann[b].end());
         }
+    }
+    // the seeing model's factors at the annuli and at the D/r0 candidates
+    std::vector<double2> ann_model(d.n_bins, make_double2(0.0, 0.0)), cand(SEEING_GRID);
+    for (int b = 1; b < d.n_bins && (double)b < r; ++b) {
+        const double rho = b / r;
+        ann_model[b] = make_double2((2.0 / M_PI) * (std::acos(rho) - rho * std::sqrt(1.0 - rho * rho)),
+                                    std::pow(rho, 5.0 / 3.0));
+    }
+    for (int i = 0; i < SEEING_GRID; ++i) {
+        const double x = std::exp(std::log(SEEING_LO) + (std::log(SEEING_HI) - std::log(SEEING_LO)) *
+                                                            ((double)i / (double)(SEEING_GRID - 1)));
+        cand[i] = make_double2(std::pow(x, 5.0 / 3.0), ch->ck / (x * x));
     }
     // The bispectrum kernel stages W and U = W - V in 16-byte copies from even
     // box columns of an even-pitched box.
@@ -512,6 +525,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {pl->tile_masks.data(), pl->tile_masks.size() * sizeof(unsigned), 0},
         {pl->units.data(), pl->units.size() * sizeof(int2), 0},
         {pl->batch_unit.data(), pl->batch_unit.size() * sizeof(int), 0},
+        {r53.data(), r53.size() * sizeof(double), 0},
+        {ann_model.data(), ann_model.size() * sizeof(double2), 0},
+        {cand.data(), cand.size() * sizeof(double2), 0},
     };
     size_t total = 0;
     for (auto& p : pcs) { p.off = total; total += align256(std::max<size_t>(p.bytes, 1)); }
@@ -549,6 +565,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.tile_masks = (const unsigned*)at(21);
     d.units = (const int2*)at(22);
     d.batch_unit = (const int*)at(23);
+    d.r53 = (const double*)at(24);
+    d.ann_model = (const double2*)at(25);
+    d.cand = (const double2*)at(26);
     *out = pl;
     return SM_OK;
 }
