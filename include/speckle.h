@@ -387,7 +387,8 @@ int sm_batch_create(int n, const sm_plan* const* plans, const int* F, const int*
 /* The shape the batch was built with (the tuned values filled in).         */
 int sm_batch_get_opts(const sm_batch* bt, sm_batch_opts* opts);
 int sm_batch_destroy(sm_batch* bt);
-/* Items in the queue, persistent CTAs of the launch, device bytes held.    */
+/* Transforms and tiles that the queue covers (SM_BATCH_GRID: 0), persistent
+ * CTAs of the launch, device bytes held.                                    */
 int sm_batch_info(const sm_batch* bt, int* n_items, int* grid, size_t* device_bytes);
 
 /* The batched transforms and bispectrum alone: spectra, flux and mean of

@@ -16,11 +16,9 @@ The fastest options of each launch per (N, R) go into the table of
 ``csrc/sm_tune.h`` (with --write), which the library compiles in: a batch
 built without options takes the fastest entry of its shape, one built with
 a launch kind but no other options takes that launch's entry.  The timings are printed as a table and, with
---write, also saved to ``profiles/autotune_batch_launch.md``.  The tile
-geometry itself (16 x 8 targets by 8 x 4 offsets per CTA) is fixed in the
-kernel; its share of computed pairs that are used is reported per shape
-(``used / computed`` from the plan), the quantity a different tile would
-change.
+--write, also saved to ``profiles/autotune_batch_launch.md``.  The tiles
+that B is stored in (16 x 8 targets by 8 x 4 offsets) are fixed; the share of
+their slots that hold a used pair is reported per shape.
 """
 from __future__ import annotations
 

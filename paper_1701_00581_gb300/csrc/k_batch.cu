@@ -11,8 +11,8 @@
 //        normalise one frame tile (the transform of k_spectra, computed by
 //        128 threads: the row transforms go to the column transforms through
 //        a per-CTA scratch tile in global memory, which stays in L2);
-//   BIS  (burst, subfield, tile):  one bispectrum tile of the subfield over
-//        all of the burst's frames (the tile body of k_bispectrum).
+//   BIS  (burst, subfield, task):  one bispectrum task of the subfield over
+//        all of the burst's frames (the body of k_bispectrum).
 //
 // A BIS item needs every frame spectrum of its subfield: each FFT item, once
 // its spectrum is stored, increments the subfield's counter (release), and a
@@ -280,15 +280,24 @@ k_batch(const __grid_constant__ BatchArgs a, const int4* __restrict__ items, int
 }
 
 // SM_BATCH_GRID: for the bursts of the batch that share one plan, one CTA
-// per (tile, subfield, burst) -- grid (n_tiles, n_sub, bursts) -- scheduled
+// per (task, subfield, burst) -- grid (n_bis_tasks, n_sub, bursts) -- scheduled
 // by the hardware like the per-stage bispectrum kernel.  The plan is a
 // by-value argument, as there, so its fields stay constant-bank operands;
 // only the bursts' buffers are looked up by blockIdx.z.
 template <int PREC, bool VCH>
 __global__ void __launch_bounds__(BT, 4) k_batch_grid(PlanDev p, const __grid_constant__ smi::BatchPtrs q) {
-    __shared__ __align__(16) float2 S[smb::staging_float2<PREC>()];
+    extern __shared__ __align__(16) float2 S[];
     const int z = blockIdx.z;
     smb::bispec_tile<PREC, VCH, false>(p, q.spec[z], q.F[z], q.B[z], blockIdx.x, blockIdx.y, S);
+}
+
+template <int PREC, bool VCH>
+cudaError_t grid_go(const PlanDev& p, const smi::BatchPtrs& q, cudaStream_t st) {
+    constexpr size_t sm = smb::staging_bytes<false>(PREC);
+    const cudaError_t e = cudaFuncSetAttribute(k_batch_grid<PREC, VCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_batch_grid<PREC, VCH><<<dim3(p.n_bis_tasks, p.n_sub, q.n), BT, sm, st>>>(p, q);
+    return cudaGetLastError();
 }
 
 size_t fft_smem_for(int N, int K) {
@@ -304,7 +313,7 @@ size_t fft_smem_for(int N, int K) {
 namespace smk {
 
 size_t batch_smem_bytes(int N, int K, int prec) {
-    const size_t bis = smb::staging_bytes(prec);
+    const size_t bis = smb::staging_bytes<false>(prec);
     const size_t fft = N > 0 ? fft_smem_for(N, K) : 0;
     return bis > fft ? bis : fft;
 }
@@ -358,19 +367,10 @@ cudaError_t launch_batch(const BatchArgs& a, int prec, int minb, const int4* ite
 }
 
 cudaError_t launch_batch_grid(const PlanDev& p, const smi::BatchPtrs& q, cudaStream_t st) {
-    const dim3 grid(p.n_tiles, p.n_sub, q.n);
     const bool vch = ((p.v_org + p.K) & 1) == 0;
-    if (p.prec == SM_FP32) {
-        if (vch) k_batch_grid<SM_FP32, true><<<grid, BT, 0, st>>>(p, q);
-        else k_batch_grid<SM_FP32, false><<<grid, BT, 0, st>>>(p, q);
-    } else if (p.prec == SM_FP16) {
-        if (vch) k_batch_grid<SM_FP16, true><<<grid, BT, 0, st>>>(p, q);
-        else k_batch_grid<SM_FP16, false><<<grid, BT, 0, st>>>(p, q);
-    } else {
-        if (vch) k_batch_grid<SM_BF16, true><<<grid, BT, 0, st>>>(p, q);
-        else k_batch_grid<SM_BF16, false><<<grid, BT, 0, st>>>(p, q);
-    }
-    return cudaGetLastError();
+    if (p.prec == SM_FP32) return vch ? grid_go<SM_FP32, true>(p, q, st) : grid_go<SM_FP32, false>(p, q, st);
+    if (p.prec == SM_FP16) return vch ? grid_go<SM_FP16, true>(p, q, st) : grid_go<SM_FP16, false>(p, q, st);
+    return vch ? grid_go<SM_BF16, true>(p, q, st) : grid_go<SM_BF16, false>(p, q, st);
 }
 
 }  // namespace smk

@@ -7,6 +7,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "sm_plan.h"
@@ -19,7 +20,8 @@ struct sm_batch {
     sm_batch_opts opts{};
     std::vector<const sm_plan*> plans;
     std::vector<int> F, frame_type, cnt_base;
-    int n_cnt = 0, n_items = 0, grid = 0, max_tiles = 0;
+    int n_cnt = 0, n_items = 0, grid = 0;
+    int n_work = 0;                     // transforms and tiles that the queue covers
     size_t smem = 0, scr_elems = 0;
     int4* d_items = nullptr;
     int* d_state = nullptr;             // [0] queue head, [1] status, [2..] per-subfield counters
@@ -36,27 +38,16 @@ namespace {
 
 size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Cost of a bispectrum tile: the CTA lasts as long as its busiest warp, which
-// runs once per offset column holding a used pair of its row.
-std::vector<int> tiles_by_cost(const sm_plan* pl) {
-    const PlanDev& d = pl->dev;
-    std::vector<int> cost(d.n_tiles, 0), order(d.n_tiles);
-    for (int t = 0; t < d.n_tiles; ++t) {
-        const int4 T = pl->tiles[t];
-        for (int q = 0; q < VBY; ++q) {
-            int cols = 0;
-            for (int kk = 0; kk < VBX; ++kk) {
-                bool any = false;
-                for (int a = 0; a < WBY && !any; ++a)
-                    for (int b = 0; b < WBX && !any; ++b)
-                        any = pair_used_host(T.x + b, T.y + a, T.z + kk, T.w + q, d.r2i, d.R * d.R);
-                cols += any;
-            }
-            cost[t] = std::max(cost[t], cols);
-        }
-    }
-    for (int t = 0; t < d.n_tiles; ++t) order[t] = t;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+// Bispectrum tasks in the order of their strips and offset blocks (the plan
+// has them costliest first).
+std::vector<int> tasks_by_place(const sm_plan* pl) {
+    std::vector<int> order(pl->dev.n_bis_tasks);
+    for (int t = 0; t < pl->dev.n_bis_tasks; ++t) order[t] = t;
+    auto key = [&](int t) {
+        const int4 a = pl->bis_tasks[2 * t], b = pl->bis_tasks[2 * t + 1];
+        return std::make_tuple(a.x, a.y / WBY, b.z);
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return key(x) < key(y); });
     return order;
 }
 
@@ -148,11 +139,11 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
     std::stable_sort(units.begin(), units.end(), [](const Unit& a, const Unit& b) { return a.pos < b.pos; });
     std::vector<std::vector<int>> order(n);
     for (int i = 0; i < n; ++i) {
-        if (opts.tile_order == 2) {
-            order[i] = tiles_by_cost(plans[i]);
+        if (opts.tile_order == 1) {
+            order[i] = tasks_by_place(plans[i]);
         } else {
-            order[i].resize(plans[i]->dev.n_tiles);
-            for (int t = 0; t < plans[i]->dev.n_tiles; ++t) order[i][t] = t;
+            order[i].resize(plans[i]->dev.n_bis_tasks);
+            for (int t = 0; t < plans[i]->dev.n_bis_tasks; ++t) order[i][t] = t;
         }
     }
     std::vector<int4> items;
@@ -169,6 +160,8 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
         }
     }
     bt->n_items = (int)items.size();
+    for (int i = 0; queued && i < n; ++i)
+        bt->n_work += plans[i]->dev.n_sub * (plans[i]->dev.n_tiles + (fused ? F[i] : 0));
 
     int old = 0;
     cudaGetDevice(&old);
@@ -191,7 +184,6 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
         return SM_ECUDA;
     }
     bt->grid = nsm * bt->blocks_per_sm;
-    for (int i = 0; i < n; ++i) bt->max_tiles = std::max(bt->max_tiles, plans[i]->dev.n_tiles);
     if (!queued) bt->grid = 0;             // a grid over (tile, subfield of every burst) per run
     bt->scr_elems = fused ? (size_t)(maxK + 1) * maxN : 0;
     if (!items.empty()) {
@@ -235,7 +227,7 @@ extern "C" int sm_batch_get_opts(const sm_batch* bt, sm_batch_opts* opts) {
 
 extern "C" int sm_batch_info(const sm_batch* bt, int* n_items, int* grid, size_t* device_bytes) {
     if (!bt) { set_error("NULL batch"); return SM_EINVAL; }
-    if (n_items) *n_items = bt->n_items;
+    if (n_items) *n_items = bt->n_work;
     if (grid) *grid = bt->grid;
     if (device_bytes)
         *device_bytes = (size_t)bt->n_items * sizeof(int4) + (size_t)(2 + bt->n_cnt) * sizeof(int) +

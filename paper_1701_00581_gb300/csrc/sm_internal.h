@@ -10,17 +10,20 @@
 
 namespace smi {
 
-// Bispectrum tile geometry (Sect. 2 / 3.2 speckle masking): a CTA owns a
-// block of WBX x WBY target frequencies w and a block of VBX x VBY offsets v.
-// Warp q of the CTA owns offset row vy0 + q; lane (wyl, gx) owns the four
-// targets (wx0 + 4 gx + j, wy0 + wyl), j = 0..3, and the eight offsets
-// (vx0 + kk, vy0 + q), kk = 0..7.  Four warps per CTA let four CTAs share
-// an SM, so warps of different tiles fill each other's idle issue slots.
+// Bispectrum tile geometry (Sect. 2 / 3.2 speckle masking): B is stored in
+// tiles, a block of WBX x WBY target frequencies w by a block of VBX x VBY
+// offsets v.  The kernel computes it in tasks (k_bispec.cu): warp q of a
+// 128-thread CTA owns offset row vy0 + q, each lane four neighbouring targets.
+// Four warps per CTA let four CTAs share an SM, so warps of different tasks
+// fill each other's idle issue slots.
 constexpr int WBX = 16, WBY = 8, VBX = 8, VBY = 4;
 constexpr int TILE_W = WBX * WBY;            // 128 targets
 constexpr int TILE_V = VBX * VBY;            // 32 offsets
 constexpr int TILE_PAIRS = TILE_W * TILE_V;  // 4096 (w, v) slots
 constexpr int BISPEC_THREADS = 32 * VBY;     // one warp per offset row
+constexpr int BIS_ROWS = 14;                 // rows of targets a task may span: more pack better (N = 128: 25 % fewer
+                                             //   columns than blocks of 8; 10 rows 15 %), and 14 rows of four CTAs
+                                             //   still fit an SM's shared memory
 static_assert(TILE_V == 32, "a tile row of offsets maps onto the 32 lanes of a warp");
 
 // Least-squares refinement partials per bispectrum tile: one per target w
@@ -38,6 +41,14 @@ constexpr double SEEING_LO = 1.0, SEEING_HI = 64.0;
 
 constexpr float FP16_SCALE = 16384.0f;       // |I_n| <= 1 -> fits half with margin
 constexpr float FP16_INV_SCALE = 1.0f / 16384.0f;
+
+// A pair whose offsets v and u = w - v both lie within R holds the same value
+// in both orders, B(u, v) = B(v, u); it is computed at the order whose v is
+// lower (then left), which empties more rows of the packed tasks than the
+// other choices.  Whether v is that order:
+__host__ __device__ inline bool pair_at_lower(int vx, int vy, int ux, int uy) {
+    return vy < uy || (vy == uy && vx <= ux);
+}
 
 // Everything a kernel needs to know about a plan, passed by value.
 struct PlanDev {
@@ -66,6 +77,14 @@ struct PlanDev {
     const int4* tiles;       // [n_tiles] wx0, wy0, vx0, vy0
     const unsigned* tile_masks;  // [n_tiles] byte q (offset row q, one warp of a tile's CTA): bit e
                                  //   set when column e holds a used pair of some target
+    const int* tile_of;      // [n_wby * n_wbx][n_vby * n_vbx] tile or -1
+    int n_vbx, n_vby;
+    // bispectrum tasks (k_bispec.cu): two int4 each -- (x of the strip, first row, vx0, vy0) and (rows; per warp
+    // a byte: first column, number of columns << 4, both even; offset block; 1 when pairs are stored twice) -- and
+    // per thread its quad, row << 2 | place in the strip, or that | INT_MIN for an idle lane
+    const int4* bis_tasks;
+    const int* bis_lanes;
+    int n_bis_tasks;
     const int* ring_start;   // [n_rings + 1]
     const int2* points;      // [n_points] (wx, wy), ring-ordered
     const int* wb_start;     // [n_wbx * n_wby + 1] CSR: tiles of each w-block

@@ -1,6 +1,7 @@
 // Plan construction: every table that depends only on the channel, built on
 // the host in double precision and uploaded once.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -104,6 +105,80 @@ int validate_channel(const sm_channel* ch) {
 
 using namespace smi;
 
+// Of four neighbouring targets and the 4 x 8 offsets of a block (bit 8 row +
+// column): the pairs that are computed for some target, and those that are
+// stored in both orders.
+struct QuadMask { unsigned compute = 0, twice = 0; };
+
+// Bispectrum tasks: per strip of 16 targets and block of offsets, each offset
+// row's quads with a pair to compute, in row order, 32 to a warp, the rows of a
+// task's four warps within BIS_ROWS of each other.
+static void pack_bis_tasks(sm_plan& pl, const std::vector<QuadMask>& quads) {
+    const PlanDev& d = pl.dev;
+    constexpr int QW = WBX / 4;
+    const int nvb = pl.n_vbx * pl.n_vby, rows_all = d.n_wby * WBY;
+    struct Task { int4 a, b; unsigned key; int lanes[BISPEC_THREADS]; };
+    std::vector<Task> tasks;
+    std::vector<std::pair<int, const QuadMask*>> list[VBY];      // (row * QW + place, masks) per offset row
+    for (int wbx = 0; wbx < d.n_wbx; ++wbx)
+        for (int vb = 0; vb < nvb; ++vb) {
+            for (int c = 0; c < VBY; ++c) list[c].clear();
+            for (int y = 0; y < rows_all; ++y) {
+                const int wb = (y / WBY) * d.n_wbx + wbx;
+                if (pl.tile_of[(size_t)wb * nvb + vb] < 0) { y |= WBY - 1; continue; }
+                const QuadMask* q = &quads[((size_t)wb * nvb + vb) * WBY * QW + (y % WBY) * QW];
+                for (int g = 0; g < QW; ++g)
+                    for (int c = 0; c < VBY; ++c)
+                        if (q[g].compute >> (8 * c) & 0xffu) list[c].push_back({y * QW + g, &q[g]});
+            }
+            size_t at[VBY] = {};
+            for (;;) {
+                int y0 = rows_all;
+                for (int c = 0; c < VBY; ++c)
+                    if (at[c] < list[c].size()) y0 = std::min(y0, list[c][at[c]].first / QW);
+                if (y0 == rows_all) break;
+                Task t = {};
+                int y1 = y0;
+                unsigned ranges = 0, most = 0, sum = 0;
+                bool twice = false;
+                for (int c = 0; c < VBY; ++c) {
+                    unsigned m = 0, both = 0;
+                    for (int l = 0; l < 32; ++l) {
+                        int& lane = t.lanes[c * 32 + l];
+                        lane = INT_MIN;                      // idle: quad 0
+                        if (at[c] >= list[c].size() || list[c][at[c]].first / QW >= y0 + BIS_ROWS) continue;
+                        const auto& q = list[c][at[c]++];
+                        lane = q.first - y0 * QW;            // row << 2 | place
+                        y1 = std::max(y1, q.first / QW);
+                        m |= q.second->compute >> (8 * c) & 0xffu;
+                        both |= q.second->twice >> (8 * c) & 0xffu;
+                    }
+                    unsigned lo = 0, hi = 0;
+                    for (unsigned e = 0; e < (unsigned)VBX; ++e)
+                        if (m >> e & 1) { if (!hi) lo = e & ~1u; hi = (e + 2) & ~1u; }
+                    ranges |= (lo | (hi - lo) << 4) << (8 * c);
+                    most = std::max(most, hi - lo);
+                    sum += hi - lo;
+                    // a pair stored twice inside the computed columns
+                    if (both & ((1u << hi) - (1u << lo))) twice = true;
+                }
+                t.a = make_int4(-d.K + WBX * wbx, y0, d.v_org + VBX * (vb % pl.n_vbx), -d.R + VBY * (vb / pl.n_vbx));
+                t.b = make_int4(y1 - y0 + 1, (int)ranges, vb, twice ? 1 : 0);
+                t.key = most * 64 + sum;
+                tasks.push_back(t);
+            }
+        }
+    // most columns first: neighbouring CTAs run the same loops, and the long
+    // tasks of a launch's last wave come early
+    std::stable_sort(tasks.begin(), tasks.end(), [](const Task& x, const Task& y) { return x.key > y.key; });
+    for (const Task& t : tasks) {
+        pl.bis_tasks.push_back(t.a);
+        pl.bis_tasks.push_back(t.b);
+        pl.bis_lanes.insert(pl.bis_lanes.end(), t.lanes, t.lanes + BISPEC_THREADS);
+    }
+    pl.dev.n_bis_tasks = (int)tasks.size();
+}
+
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
@@ -205,6 +280,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     const int nwb = d.n_wbx * d.n_wby, nvb = pl->n_vbx * pl->n_vby;
     pl->tile_of.assign((size_t)nwb * nvb, -1);
     std::vector<int> wb_count(nwb, 0);
+    std::vector<QuadMask> quads((size_t)nwb * nvb * WBY * (WBX / 4));
+    d.n_vbx = pl->n_vbx;
+    d.n_vby = pl->n_vby;
     long long npairs = 0;
     for (int wby = 0; wby < d.n_wby; ++wby)
         for (int wbx = 0; wbx < d.n_wbx; ++wbx) {
@@ -217,14 +295,22 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
                     // of the bispectrum CTA) the columns e holding one
                     long long cnt = 0;
                     unsigned mask = 0;
+                    const int vb = vby * pl->n_vbx + vbx;
+                    QuadMask* const qm = &quads[((size_t)wb * nvb + vb) * WBY * (WBX / 4)];
                     for (int a = 0; a < WBY; ++a)
                         for (int b = 0; b < WBX; ++b)
                             for (int c = 0; c < VBY; ++c)
-                                for (int e = 0; e < VBX; ++e)
-                                    if (pair_used_host(wx0 + b, wy0 + a, vx0 + e, vy0 + c, r2i, R * R)) {
-                                        ++cnt;
-                                        mask |= 1u << (8 * c + e);
-                                    }
+                                for (int e = 0; e < VBX; ++e) {
+                                    const int wx = wx0 + b, wy = wy0 + a, vx = vx0 + e, vy = vy0 + c;
+                                    if (!pair_used_host(wx, wy, vx, vy, r2i, R * R)) continue;
+                                    ++cnt;
+                                    mask |= 1u << (8 * c + e);
+                                    QuadMask& m = qm[a * (WBX / 4) + b / 4];
+                                    const int ux = wx - vx, uy = wy - vy;
+                                    const bool both = ux * ux + uy * uy <= R * R;
+                                    if (both) m.twice |= 1u << (8 * c + e);
+                                    if (!both || pair_at_lower(vx, vy, ux, uy)) m.compute |= 1u << (8 * c + e);
+                                }
                     if (cnt == 0) continue;
                     npairs += cnt;
                     pl->tile_of[(size_t)wb * nvb + vby * pl->n_vbx + vbx] = (int)pl->tiles.size();
@@ -234,6 +320,8 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
                 }
         }
     d.n_tiles = (int)pl->tiles.size();
+
+    pack_bis_tasks(*pl, quads);
 
     // seeing cubes (Sect. 3.1): non-overlapping N x N tiles from the image
     // origin, i.e. the full-size subfields whose corner lies on the N grid
@@ -528,6 +616,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {r53.data(), r53.size() * sizeof(double), 0},
         {ann_model.data(), ann_model.size() * sizeof(double2), 0},
         {cand.data(), cand.size() * sizeof(double2), 0},
+        {pl->tile_of.data(), pl->tile_of.size() * sizeof(int), 0},
+        {pl->bis_tasks.data(), pl->bis_tasks.size() * sizeof(int4), 0},
+        {pl->bis_lanes.data(), pl->bis_lanes.size() * sizeof(int), 0},
     };
     size_t total = 0;
     for (auto& p : pcs) { p.off = total; total += align256(std::max<size_t>(p.bytes, 1)); }
@@ -568,6 +659,9 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.r53 = (const double*)at(24);
     d.ann_model = (const double2*)at(25);
     d.cand = (const double2*)at(26);
+    d.tile_of = (const int*)at(27);
+    d.bis_tasks = (const int4*)at(28);
+    d.bis_lanes = (const int*)at(29);
     *out = pl;
     return SM_OK;
 }

@@ -13,6 +13,8 @@ struct sm_plan {
     std::vector<int4> subs;
     std::vector<int4> tiles;
     std::vector<unsigned> tile_masks;   // [tile] byte q: offset columns of row q holding a used pair
+    std::vector<int4> bis_tasks;        // bispectrum tasks (sm_internal.h)
+    std::vector<int> bis_lanes;
     std::vector<int> tile_of;        // [w-block][v-block] -> tile id or -1
     int n_vbx = 0, n_vby = 0;
     std::vector<int> wb_start, wb_tiles;

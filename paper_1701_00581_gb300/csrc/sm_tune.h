@@ -14,15 +14,15 @@ struct TuneEntry {
 
 // BEGIN TABLE (autotune.py)
 constexpr TuneEntry kTune[] = {
-    {256, 24, 4, 4, 1, 1, 109.7350},
-    {256, 24, 2, 4, 2, 1, 108.4027},
-    {256, 24, 2, 4, 3, 1, 108.5971},
-    {128, 16, 4, 4, 1, 2, 14.0166},
-    {128, 16, 2, 4, 2, 2, 14.2122},
-    {128, 16, 2, 4, 3, 1, 14.1201},
-    {64, 8, 4, 3, 1, 1, 0.0238},
-    {64, 8, 2, 3, 2, 2, 0.0218},
-    {64, 8, 2, 4, 3, 1, 0.0209},
+    {256, 24, 4, 4, 1, 1, 100.4666},
+    {256, 24, 2, 4, 2, 1, 97.5258},
+    {256, 24, 2, 4, 3, 1, 93.4097},
+    {128, 16, 4, 3, 1, 2, 14.0158},
+    {128, 16, 2, 4, 2, 2, 11.8864},
+    {128, 16, 2, 4, 3, 1, 11.5035},
+    {64, 8, 4, 4, 1, 1, 0.0222},
+    {64, 8, 2, 3, 2, 1, 0.0216},
+    {64, 8, 2, 4, 3, 1, 0.0188},
 };
 // END TABLE
 
