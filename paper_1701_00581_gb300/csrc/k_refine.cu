@@ -23,6 +23,7 @@
 // k_refine_gather: eight CTAs per subfield, one warp per recursion point,
 // sums the point's partials from the plan's list along a fixed tree and
 // renormalises.  No atomics: the result does not depend on scheduling.
+#include <cfloat>
 #include "sm_internal.h"
 
 namespace {
@@ -195,6 +196,20 @@ k_refine_tiles(PlanDev p, const float2* __restrict__ B, const float* __restrict_
     }
 }
 
+// (hi, lo) += (h, l) as a pair of floats with about 48 significant bits
+// (Knuth's two-sum, then the renormalising fast two-sum).
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float h, float l) {
+    const float s = __fadd_rn(hi, h), v = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(h, v)), __fadd_rn(lo, l));
+    hi = __fadd_rn(s, e);
+    lo = __fsub_rn(e, __fsub_rn(hi, s));
+}
+
+// A warp per point; the sums run on pairs of floats, and the normalisation in
+// FP64 is done for up to 32 of the warp's points at once, one per lane: GB300's
+// FP64 unit takes 16 cycles per warp instruction whatever its lanes do, and a
+// root and two divisions for one lane were most of the kernel's time
+// (63 subfields of 128^2, R = 16: 497 -> 62 us a sweep).
 __global__ void __launch_bounds__(RG_THREADS)
 k_refine_gather(PlanDev p, const float2* __restrict__ partials, double2* __restrict__ z) {
     const int sl = blockIdx.x, lane = threadIdx.x & 31;
@@ -203,29 +218,54 @@ k_refine_gather(PlanDev p, const float2* __restrict__ partials, double2* __restr
     const int K = p.K, pitch = p.box_pitch;
     double2* zs = z + (size_t)sl * p.hb_rows * pitch;
     const float2* part = partials + (size_t)sl * p.n_tiles * REF_SLOTS;
-    for (int pi = gwarp; pi < p.n_points; pi += nwarp) {
-        double sx = 0.0, sy = 0.0;
-        const int a0 = p.ref_start[pi], a1 = p.ref_start[pi + 1];
-        // two entries per lane per step, both loads in flight together
-        for (int a = a0 + lane; a < a1; a += 64) {
-            const bool two = a + 32 < a1;
-            const int e0 = p.ref_idx[a];
-            const int e1 = two ? p.ref_idx[a + 32] : 0;
-            const float2 c0 = part[e0 & 0x7fffffff];
-            const float2 c1 = two ? part[e1 & 0x7fffffff] : make_float2(0.f, 0.f);
-            sx += (double)c0.x + (double)c1.x;
-            sy += (e0 < 0 ? -(double)c0.y : (double)c0.y) + (e1 < 0 ? -(double)c1.y : (double)c1.y);
-        }
+    for (int p0 = gwarp; p0 < p.n_points; p0 += 32 * nwarp) {
+        float kx = 0.f, kxl = 0.f, ky = 0.f, kyl = 0.f;       // the sum of this lane's point
+        for (int k = 0; k < 32 && p0 + k * nwarp < p.n_points; ++k) {
+            const int pi = p0 + k * nwarp;
+            float sx = 0.f, sxl = 0.f, sy = 0.f, syl = 0.f;
+            const int a0 = p.ref_start[pi], a1 = p.ref_start[pi + 1];
+            // four entries per lane per step, their loads in flight together
+            for (int a = a0 + lane; a < a1; a += 128) {
+                int e[4];
+                float2 c[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+                for (int i = 0; i < 4; ++i) e[i] = a + 32 * i < a1 ? p.ref_idx[a + 32 * i] : 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    c[i] = a + 32 * i < a1 ? part[e[i] & 0x7fffffff] : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    pair_add(sx, sxl, c[i].x, 0.f);
+                    pair_add(sy, syl, e[i] < 0 ? -c[i].y : c[i].y, 0.f);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float hx = __shfl_xor_sync(0xffffffffu, sx, o), lx = __shfl_xor_sync(0xffffffffu, sxl, o);
+                const float hy = __shfl_xor_sync(0xffffffffu, sy, o), ly = __shfl_xor_sync(0xffffffffu, syl, o);
+                pair_add(sx, sxl, hx, lx);
+                pair_add(sy, syl, hy, ly);
+            }
+            if (lane == k) kx = sx, kxl = sxl, ky = sy, kyl = syl;
         }
-        if (lane == 0) {
-            const double n = sqrt(sx * sx + sy * sy);
+        const int pi = p0 + lane * nwarp;
+        if (pi < p.n_points) {
+            double x = (double)kx + (double)kxl, y = (double)ky + (double)kyl;
+            // an infinite term or a sum beyond the range of a float, which a pair
+            // of floats turns into NaN: this point's sum in FP64 after all
+            if (!(fabs(x) + fabs(y) < DBL_MAX)) {
+                x = y = 0.0;
+                for (int a = p.ref_start[pi]; a < p.ref_start[pi + 1]; ++a) {
+                    const int e = p.ref_idx[a];
+                    const float2 c = part[e & 0x7fffffff];
+                    x += (double)c.x;
+                    y += (double)(e < 0 ? -c.y : c.y);
+                }
+            }
+            const double n = sqrt(x * x + y * y);
             if (n > 0.0) {
                 const int2 w = p.points[pi];
-                const double2 zz = make_double2(sx / n, sy / n);
+                const double2 zz = make_double2(x / n, y / n);
                 zs[w.y * pitch + w.x + K] = zz;
                 if (w.y == 0) zs[-w.x + K] = make_double2(zz.x, -zz.y);
             }
