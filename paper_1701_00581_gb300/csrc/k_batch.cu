@@ -89,7 +89,7 @@ __device__ __forceinline__ void fft_item(const PlanDev& p, const TIn* __restrict
     const int4 sb = p.subs[s];
     const int x0 = sb.x, y0 = sb.y, w = sb.z, h = sb.w;
     for (int i = tid; i < N; i += BT) {
-        stw[i] = p.tw[i];
+        stw[i] = p.tw[smf::step_root<N>(i)];
         swx[i] = p.winx[(size_t)s * N + i];
         swy[i] = p.winy[(size_t)s * N + i];
     }

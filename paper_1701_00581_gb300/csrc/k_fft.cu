@@ -17,28 +17,39 @@ using smf::load_sample;
 using smf::Split;
 using smf::store_spec;
 
-// 32 groups of 16 threads for N >= 128 (one CTA per SM fits in shared memory,
-// so latency is hidden by warps within the CTA).
-template <int N> struct SpecThreads { static constexpr int T = N >= 128 ? 512 : 256; };
-
-// Thread groups of the four-step transform: G threads per transform.
-template <int N> struct Grp {
+// Thread groups of the four-step transform: G threads per transform, each
+// forming U groups of P outputs.  TB: the exchange tile's elements (it holds a
+// row for the inverse; groups of 8 threads start half the banks apart).
+template <int N, int THREADS, int OUT, int RESIDENT> struct Grp {
     static constexpr int P = Split<N>::P, Q = Split<N>::Q;
-    static constexpr int G = P > Q ? P : Q;
-    static constexpr int NG = SpecThreads<N>::T / G;                 // groups per CTA
-    static constexpr int TB = (Q * (P + 1) > N ? Q * (P + 1) : N);   // exchange buffer
+    static constexpr int T = THREADS, U = OUT, G = Q / OUT, CTAS = RESIDENT;
+    static constexpr int NG = T / G;
+    static constexpr int TB0 = Q * (P + 1) > N ? Q * (P + 1) : N;
+    static constexpr int TB = G == 8 ? (TB0 + 7) / 16 * 16 + 8 : TB0;
+    static_assert(G >= P && (N / 2) % NG == 0, "a thread per first-stage input, whole rounds of row pairs");
 };
 
-// scratch area (float2): the groups' exchange tiles
-template <int N>
-__host__ __device__ constexpr int scratch_elems() { return Grp<N>::NG * Grp<N>::TB; }
-__host__ __device__ constexpr int scratch_elems_rt(int N) {
-    return N == 64 ? scratch_elems<64>() : (N == 128 ? scratch_elems<128>() : scratch_elems<256>());
-}
+// Spectra.  N = 256: 32 groups of 16 threads; one CTA per SM fits in shared
+// memory, so latency is hidden by the warps within it.  N = 128: groups of 8
+// threads with two output sets each, so that no lane idles in the first stage.
+// Smaller transforms run several CTAs to an SM, which hide each other's
+// barriers and chains.
+template <int N> struct SpecGrp;
+template <> struct SpecGrp<64> : Grp<64, 128, 1, 6> {};
+template <> struct SpecGrp<128> : Grp<128, 128, 2, 3> {};
+template <> struct SpecGrp<256> : Grp<256, 512, 1, 1> {};
+// N = 64 with few tiles: twice the threads per tile.  100 tiles: 5.3 us against
+// 6.6 with 128 threads; 400 (a wave of three per SM): 7.4 against 8.7; 500:
+// 11.4 against 9.7; 36100: 471 against 376.
+struct SpecGrpFew : Grp<64, 256, 1, 3> {};
 
+// Inverse: one CTA per subfield, as many threads as the rows keep busy.
+template <int N> struct InvGrp : Grp<N, N >= 128 ? 512 : 256, 1, 1> {};
+
+template <typename GP>
 __host__ __device__ constexpr size_t fft_smem(int N, int K) {
     return (size_t)(K + 1) * (N + 1) * sizeof(float2)        // column buffer
-           + (size_t)scratch_elems_rt(N) * sizeof(float2)    // scratch
+           + (size_t)GP::NG * GP::TB * sizeof(float2)        // the groups' exchange tiles
            + (size_t)N * sizeof(float2)                      // twiddles
            + (size_t)(K + 1) * sizeof(float2)                // window transform
            + (size_t)2 * N * sizeof(float)                   // windows
@@ -49,18 +60,23 @@ __host__ __device__ constexpr size_t fft_smem(int N, int K) {
 // row by row (two real rows per complex transform), the windowed mean mu is
 // read off the row transforms' DC terms, mu * window is removed through the
 // window's own transform, and the K+1 non-negative columns are transformed.
-template <int N, typename TIn, int PREC>
-__global__ void __launch_bounds__(SpecThreads<N>::T, 1)
+// Bound by issue and shared-memory wavefronts, not by HBM (a quarter of the
+// copy rate at most): rotations by sixteenth roots are constants of the code,
+// the four-step roots are read in lane order, the row pairs are taken apart by
+// shuffles and the mean goes in the columns' load.  100 frames of uint16:
+// 304 subfields of 256^2 5.36 -> 4.47 ms, 225 of 128^2 2.56 -> 0.97 ms, 361 of
+// 64^2 0.45 -> 0.38 ms, one of 64^2 6.2 -> 5.7 us.
+template <typename GP, int N, typename TIn, int PREC>
+__global__ void __launch_bounds__(GP::T, GP::CTAS)
 k_spectra(PlanDev p, const TIn* __restrict__ frames, int F, int sub0, void* __restrict__ spec,
           float* __restrict__ flux, float* __restrict__ mu) {
-    using GP = Grp<N>;
-    constexpr int P = GP::P, Q = GP::Q, G = GP::G, NG = GP::NG, TB = GP::TB;
-    constexpr int TS = SpecThreads<N>::T, WS = TS / 32;
+    constexpr int P = GP::P, Q = GP::Q, G = GP::G, NG = GP::NG, TB = GP::TB, U = GP::U;
+    constexpr int TS = GP::T, WS = TS / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     const int K1 = p.K + 1, CP = N + 1;
     float2* C = reinterpret_cast<float2*>(smem);
     float2* scratch = C + (size_t)K1 * CP;
-    float2* stw = scratch + scratch_elems<N>();
+    float2* stw = scratch + NG * TB;
     float2* swf = stw + N;
     float* swx = reinterpret_cast<float*>(swf + K1);
     float* swy = swx + N;
@@ -87,48 +103,59 @@ k_spectra(PlanDev p, const TIn* __restrict__ frames, int F, int sub0, void* __re
             asm volatile("prefetch.global.L2 [%0];" :: "l"(fb + (off > lo ? off : lo)));
         }
     }
-    for (int i = tid; i < N; i += TS) {
-        stw[i] = p.tw[i];
-        swx[i] = p.winx[(size_t)s * N + i];
-        swy[i] = p.winy[(size_t)s * N + i];
-    }
-    for (int i = tid; i < K1; i += TS) swf[i] = p.winft[(size_t)s * K1 + i];
-    __syncthreads();
-
     const TIn* fr = frames + (size_t)f * p.H * p.W + (size_t)y0 * p.W + x0;
-    // row transforms: group grp of round r handles rows 2(r NG + grp), +1
+    // row transforms: group grp of round r handles rows 2(r NG + grp), +1; a
+    // round's samples are on their way while the round before is taken apart
     float raw[2][Q];
     auto fetch = [&](int pr) {
         const int y1 = 2 * pr, y2 = y1 + 1;
 #pragma unroll
         for (int n2 = 0; n2 < Q; ++n2) {
             const int x = g + P * n2;
-            const bool inx = g < P && x < w;
+            const bool inx = (G == P || g < P) && x < w;
             raw[0][n2] = inx && y1 < h ? load_sample(fr + (size_t)y1 * p.W + x) : 0.f;
             raw[1][n2] = inx && y2 < h ? load_sample(fr + (size_t)y2 * p.W + x) : 0.f;
         }
     };
+    fetch(grp);
+    for (int i = tid; i < N; i += TS) {
+        stw[i] = p.tw[smf::step_root<N>(i)];
+        swx[i] = p.winx[(size_t)s * N + i];
+        swy[i] = p.winy[(size_t)s * N + i];
+    }
+    for (int i = tid; i < K1; i += TS) swf[i] = p.winft[(size_t)s * K1 + i];
+    __syncthreads();
+
+    const double wsum = tid == 0 ? p.winsum[s] : 0.0;
+#pragma unroll 1
     for (int pr0 = 0; pr0 < N / 2; pr0 += NG) {
-        fetch(pr0 + grp);
         const int pr = pr0 + grp, y1 = 2 * pr, y2 = y1 + 1;
-        float2 v[Q], X[P];
+        float2 v[Q], X[U * P];
 #pragma unroll
         for (int n2 = 0; n2 < Q; ++n2) {
             const float wx = swx[(g + P * n2) & (N - 1)];
             v[n2] = make_float2(wx * swy[y1] * raw[0][n2], wx * swy[y2] * raw[1][n2]);
         }
-        four_step<N, false>(v, X, T, stw, g);
-        if (g < Q) {
+        four_step<N, false, U>(v, X, T, stw, g);
+        if (pr0 + NG < N / 2) fetch(pr + NG);
+        // the two rows' transforms from X(kx) and X(N - kx), which is the
+        // value [U - 1 - u][P - 1 - k1] of lane G - g (lane 0: its own, one
+        // place on); kx <= K < N / 2
+        const int partner = (lane & ~(G - 1)) | ((G - g) & (G - 1));
 #pragma unroll
-            for (int k1 = 0; k1 < P; ++k1) T[g + Q * k1] = X[k1];
-        }
-        __syncwarp();
-        for (int kx = g; kx < K1; kx += G) {
-            const float2 za = T[kx], zb = T[(N - kx) & (N - 1)];
-            C[kx * CP + y1] = make_float2(0.5f * (za.x + zb.x), 0.5f * (za.y - zb.y));
-            C[kx * CP + y2] = make_float2(0.5f * (za.y + zb.y), -0.5f * (za.x - zb.x));
-        }
-        __syncwarp();
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k1 = 0; k1 < P / 2; ++k1) {
+                if (G * u + Q * k1 >= K1) break;
+                const float2 za = X[u * P + k1], m = X[(U - 1 - u) * P + P - 1 - k1];
+                float2 zb = make_float2(__shfl_sync(0xffffffffu, m.x, partner), __shfl_sync(0xffffffffu, m.y, partner));
+                if (g == 0) zb = u > 0 ? X[(U - u) % U * P + P - 1 - k1] : X[(P - k1) % P];
+                const int kx = g + G * u + Q * k1;
+                if (kx < K1) {
+                    C[kx * CP + y1] = make_float2(0.5f * (za.x + zb.x), 0.5f * (za.y - zb.y));
+                    C[kx * CP + y2] = make_float2(0.5f * (za.y + zb.y), -0.5f * (za.x - zb.x));
+                }
+            }
     }
     __syncthreads();
 
@@ -144,40 +171,47 @@ k_spectra(PlanDev p, const TIn* __restrict__ frames, int F, int sub0, void* __re
     __syncthreads();
     if (tid == 0) {
         double tot = 0.0;
+#pragma unroll
         for (int i = 0; i < (N < TS ? N : TS) / 32; ++i) tot += red[i];
-        const double wsum = p.winsum[s];
         const float m = (float)(tot / wsum);
-        const double fl = (double)m * wsum;
-        red[WS] = fl;                                  // flux, then its reciprocal and the mean
-        reinterpret_cast<float*>(red + WS + 1)[0] = (float)(1.0 / fl);
         reinterpret_cast<float*>(red + WS + 1)[1] = m;
     }
     __syncthreads();
     const float mean = reinterpret_cast<const float*>(red + WS + 1)[1];
-    // remove mean * window: row transform of w_x(x) w_y(y) mu is mu w_y(y) Wx(kx)
-    // (a warp per column, lanes along it: no index division per element)
-    for (int kx = warp; kx < K1; kx += WS) {
-        const float2 wf = swf[kx];
-        for (int y = lane; y < h; y += 32) {
-            const float a = mean * swy[y];
-            float2& c = C[kx * CP + y];
-            c.x -= a * wf.x;
-            c.y -= a * wf.y;
-        }
+    if (tid == 0) {
+        const double fl = (double)mean * wsum;
+        red[WS] = fl;                                  // flux, then its reciprocal
+        reinterpret_cast<float*>(red + WS + 1)[0] = (float)(1.0 / fl);
     }
-    __syncthreads();
 
-    // column transforms of kx = 0..K (groups past K transform column K and drop it)
+    // column transforms of kx = 0..K (groups past K transform column K and
+    // drop it), with mean * window removed on the way in: the row transform of
+    // w_x(x) w_y(y) mu is mu w_y(y) Wx(kx)
     for (int c0 = 0; c0 < K1; c0 += NG) {
         const int kx = c0 + grp;
         const int kc = kx < K1 ? kx : K1 - 1;
-        float2 v[Q], X[P];
+        const float2 wf = swf[kc];
+        float2 v[Q], X[U * P];
 #pragma unroll
-        for (int n2 = 0; n2 < Q; ++n2) v[n2] = g < P ? C[kc * CP + g + P * n2] : make_float2(0.f, 0.f);
-        four_step<N, false>(v, X, T, stw, g);
-        if (kx < K1 && g < Q) {
+        for (int n2 = 0; n2 < Q; ++n2) {
+            const int y = g + P * n2;
+            float2 c = make_float2(0.f, 0.f);
+            if (G == P || g < P) {
+                c = C[kc * CP + y];
+                if (y < h) {
+                    const float a = mean * swy[y];
+                    c.x -= a * wf.x;
+                    c.y -= a * wf.y;
+                }
+            }
+            v[n2] = c;
+        }
+        four_step<N, false, U>(v, X, T, stw, g);
+        if (kx < K1) {
 #pragma unroll
-            for (int k1 = 0; k1 < P; ++k1) C[kx * CP + g + Q * k1] = X[k1];
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int k1 = 0; k1 < P; ++k1) C[kx * CP + g + G * u + Q * k1] = X[u * P + k1];
         }
         __syncwarp();
     }
@@ -227,17 +261,18 @@ __device__ __forceinline__ float scaled(float a, double v) {
 // (warp-wide radix-2 passes in shared memory, FP64 products and a serial sum
 // over the frames before).
 template <int N>
-__global__ void __launch_bounds__(SpecThreads<N>::T, 1)
+__global__ void __launch_bounds__(InvGrp<N>::T, InvGrp<N>::CTAS)
 k_inverse(PlanDev p, int F, int sub0, const float* __restrict__ A, const double2* __restrict__ z,
           const float* __restrict__ flux, const float* __restrict__ mu, float* __restrict__ rec) {
-    using GP = Grp<N>;
+    using GP = InvGrp<N>;
     constexpr int P = GP::P, Q = GP::Q, G = GP::G, NG = GP::NG, TB = GP::TB;
-    constexpr int TS = SpecThreads<N>::T, WS = TS / 32;
+    constexpr int TS = GP::T, WS = TS / 32;
+    static_assert(GP::U == 1, "one output set per thread");
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, K1 = K + 1, CP = N + 1;
     float2* C = reinterpret_cast<float2*>(smem);
     float2* scratch = C + (size_t)K1 * CP;
-    float2* stw = scratch + scratch_elems<N>();
+    float2* stw = scratch + NG * TB;
     float* swx = reinterpret_cast<float*>(stw + N + K1);
     float* swy = swx + N;
     double* red = reinterpret_cast<double*>(swy + N);
@@ -247,7 +282,7 @@ k_inverse(PlanDev p, int F, int sub0, const float* __restrict__ A, const double2
     const int grp = tid / G, g = tid - grp * G;
     float2* T = scratch + grp * TB;
     for (int i = tid; i < N; i += TS) {
-        stw[i] = p.tw[i];
+        stw[i] = p.tw[smf::step_root<N>(i)];
         swx[i] = p.winx[(size_t)s * N + i];
         swy[i] = p.winy[(size_t)s * N + i];
     }
@@ -332,18 +367,18 @@ k_inverse(PlanDev p, int F, int sub0, const float* __restrict__ A, const double2
     }
 }
 
-template <int N>
+template <typename GP, int N>
 cudaError_t spectra_n(const PlanDev& p, const void* frames, int frame_type, int F, int sub0,
                       int nsub, void* spec, float* flux, float* mu, cudaStream_t st) {
-    const size_t sm = fft_smem(N, p.K);
+    const size_t sm = fft_smem<GP>(N, p.K);
     dim3 grid(nsub, F);
     cudaError_t e = cudaSuccess;
 #define SM_LAUNCH(TIN, PREC)                                                                    \
     do {                                                                                        \
-        e = cudaFuncSetAttribute(k_spectra<N, TIN, PREC>,                                       \
+        e = cudaFuncSetAttribute(k_spectra<GP, N, TIN, PREC>,                                       \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);         \
         if (e != cudaSuccess) return e;                                                         \
-        k_spectra<N, TIN, PREC><<<grid, SpecThreads<N>::T, sm, st>>>(                                 \
+        k_spectra<GP, N, TIN, PREC><<<grid, GP::T, sm, st>>>(                                         \
             p, reinterpret_cast<const TIN*>(frames), F, sub0, spec, flux, mu);                  \
     } while (0)
     if (frame_type == SM_U16) {
@@ -362,27 +397,43 @@ cudaError_t spectra_n(const PlanDev& p, const void* frames, int frame_type, int 
 template <int N>
 cudaError_t inverse_n(const PlanDev& p, int F, int sub0, int nsub, const float* A, const double2* z,
                       const float* flux, const float* mu, float* rec, cudaStream_t st) {
-    const size_t sm = fft_smem(N, p.K);
+    const size_t sm = fft_smem<InvGrp<N>>(N, p.K);
     cudaError_t e = cudaFuncSetAttribute(k_inverse<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
     if (e != cudaSuccess) return e;
-    k_inverse<N><<<nsub, SpecThreads<N>::T, sm, st>>>(p, F, sub0, A, z, flux, mu, rec);
+    k_inverse<N><<<nsub, InvGrp<N>::T, sm, st>>>(p, F, sub0, A, z, flux, mu, rec);
     return cudaGetLastError();
+}
+
+// Tiles up to which a 64 x 64 tile gets 256 threads instead of 128: one wave
+// of them.
+long long few_tiles() {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (long long)SpecGrpFew::CTAS * sms;
 }
 
 }  // namespace
 
 namespace smk {
 
-size_t spectra_smem_bytes(int N, int K) { return fft_smem(N, K); }
+size_t spectra_smem_bytes(int N, int K) {
+    return N == 64    ? fft_smem<InvGrp<64>>(N, K)
+           : N == 128 ? fft_smem<InvGrp<128>>(N, K)
+                      : fft_smem<InvGrp<256>>(N, K);
+}
 
 cudaError_t launch_spectra(const smi::PlanDev& p, const void* frames, int frame_type, int F,
                            int sub0, int nsub, void* spec, float* flux, float* mu,
                            cudaStream_t st) {
     switch (p.N) {
-        case 64: return spectra_n<64>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
-        case 128: return spectra_n<128>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
-        case 256: return spectra_n<256>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
+        case 64:
+            if ((long long)nsub * F <= few_tiles())
+                return spectra_n<SpecGrpFew, 64>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
+            return spectra_n<SpecGrp<64>, 64>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
+        case 128: return spectra_n<SpecGrp<128>, 128>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
+        case 256: return spectra_n<SpecGrp<256>, 256>(p, frames, frame_type, F, sub0, nsub, spec, flux, mu, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -11,9 +11,8 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// In-register radix-2 FFT of length L (decimation in time, bit-reversed
-// input order resolved at compile time).  tw[m] = exp(-2 pi i m / N) for the
-// transform size N of the kernel; W_L^k = tw[k N / L].  INV conjugates.
+// In-register radix-2 FFT of length 8 or 16 (decimation in time, bit-reversed
+// input order resolved at compile time).  INV conjugates.
 __host__ __device__ constexpr int bitrev(int i, int bits) {
     int r = 0;
     for (int b = 0; b < bits; ++b) r |= ((i >> b) & 1) << (bits - 1 - b);
@@ -21,9 +20,45 @@ __host__ __device__ constexpr int bitrev(int i, int bits) {
 }
 __host__ __device__ constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n / 2); }
 
-template <int L, int N, bool INV>
-__device__ __forceinline__ void reg_fft(float2 (&v)[L], const float2* tw) {
+// b W_16^E (E < 8), the conjugate for INV: the factors are constants of the
+// code, so the eighth roots cost two products and the quarter root none.
+template <int E, bool INV>
+__device__ __forceinline__ float2 rotate16(float2 b) {
+    constexpr float h = 0.70710678118654752440f;     // cos(pi/4)
+    constexpr float c = 0.92387953251128675613f;     // cos(pi/8)
+    constexpr float s = 0.38268343236508977173f;     // sin(pi/8)
+    if constexpr (E == 0) return b;
+    else if constexpr (E == 4) return INV ? make_float2(-b.y, b.x) : make_float2(b.y, -b.x);
+    else if constexpr (E == 2)
+        return INV ? make_float2(h * (b.x - b.y), h * (b.x + b.y)) : make_float2(h * (b.x + b.y), h * (b.y - b.x));
+    else if constexpr (E == 6)
+        return INV ? make_float2(-h * (b.x + b.y), h * (b.x - b.y)) : make_float2(h * (b.y - b.x), -h * (b.x + b.y));
+    else {
+        constexpr float wx = E == 1 ? c : E == 3 ? s : E == 5 ? -s : -c;
+        constexpr float wy = (E == 1 ? -s : E == 3 ? -c : E == 5 ? -c : -s) * (INV ? -1.f : 1.f);
+        return cmul(b, make_float2(wx, wy));
+    }
+}
+
+// One butterfly level of the FFT below: blocks of LEN, factor W_LEN^J.
+template <int L, int LEN, int J, bool INV>
+__device__ __forceinline__ void fft_level(float2 (&v)[L]) {
+    if constexpr (J < LEN / 2) {
+#pragma unroll
+        for (int i = 0; i < L; i += LEN) {
+            const float2 a = v[i + J];
+            const float2 t = rotate16<J * (16 / LEN), INV>(v[i + J + LEN / 2]);
+            v[i + J] = make_float2(a.x + t.x, a.y + t.y);
+            v[i + J + LEN / 2] = make_float2(a.x - t.x, a.y - t.y);
+        }
+        fft_level<L, LEN, J + 1, INV>(v);
+    }
+}
+
+template <int L, bool INV>
+__device__ __forceinline__ void reg_fft(float2 (&v)[L]) {
     constexpr int LB = ilog2(L);
+    static_assert(L == 8 || L == 16, "rotations are sixteenth roots");
 #pragma unroll
     for (int i = 0; i < L; ++i) {
         const int j = bitrev(i, LB);
@@ -33,23 +68,10 @@ __device__ __forceinline__ void reg_fft(float2 (&v)[L], const float2* tw) {
             v[j] = t;
         }
     }
-#pragma unroll
-    for (int len = 2; len <= L; len <<= 1) {
-        const int half = len / 2;
-#pragma unroll
-        for (int j = 0; j < half; ++j) {
-            float2 w = tw[j * (N / len)];
-            if (INV) w.y = -w.y;
-#pragma unroll
-            for (int i = 0; i < L; i += len) {
-                const float2 a = v[i + j];
-                const float2 b = v[i + j + half];
-                const float2 t = j == 0 ? b : cmul(b, w);
-                v[i + j] = make_float2(a.x + t.x, a.y + t.y);
-                v[i + j + half] = make_float2(a.x - t.x, a.y - t.y);
-            }
-        }
-    }
+    fft_level<L, 2, 0, INV>(v);
+    fft_level<L, 4, 0, INV>(v);
+    fft_level<L, 8, 0, INV>(v);
+    if constexpr (L == 16) fft_level<L, 16, 0, INV>(v);
 }
 
 // Four-step split of an N-point transform: N = P * Q, thread n1 < P of a
@@ -60,24 +82,38 @@ template <> struct Split<64> { static constexpr int P = 8, Q = 8; };
 template <> struct Split<128> { static constexpr int P = 8, Q = 16; };
 template <> struct Split<256> { static constexpr int P = 16, Q = 16; };
 
-template <int N, bool INV>
-__device__ __forceinline__ void four_step(float2 (&v)[Split<N>::Q], float2 (&out)[Split<N>::P],
+// Entry i = k2 P + g of the four-step table: exp(-2 pi i g k2 / N), so that a
+// group's lanes read neighbouring words (in the plan's order W_N^j the reads
+// of stage k2 would share gcd(k2, 16) banks and cost as much as the exchange).
+template <int N>
+__device__ __forceinline__ int step_root(int i) { return (i % Split<N>::P) * (i / Split<N>::P); }
+
+// U: outputs of the second stage per thread, of G = Q / U threads: output
+// k = g + G u + Q k1 is out[u P + k1].
+template <int N, bool INV, int U = 1>
+__device__ __forceinline__ void four_step(float2 (&v)[Split<N>::Q], float2 (&out)[U * Split<N>::P],
                                           float2* T, const float2* tw, int g) {
-    constexpr int P = Split<N>::P, Q = Split<N>::Q;
-    if (g < P) {
-        reg_fft<Q, N, INV>(v, tw);
+    constexpr int P = Split<N>::P, Q = Split<N>::Q, G = Q / U;
+    if (G == P || g < P) {
+        reg_fft<Q, INV>(v);
 #pragma unroll
         for (int k2 = 0; k2 < Q; ++k2) {
-            float2 w = tw[g * k2];
+            float2 w = tw[k2 * P + g];
             if (INV) w.y = -w.y;
             T[k2 * (P + 1) + g] = k2 == 0 ? v[k2] : cmul(v[k2], w);
         }
     }
     __syncwarp();
-    if (g < Q) {
+    if (g < G) {
 #pragma unroll
-        for (int n1 = 0; n1 < P; ++n1) out[n1] = T[g * (P + 1) + n1];
-        reg_fft<P, N, INV>(out, tw);
+        for (int u = 0; u < U; ++u) {
+            float2 o[P];
+#pragma unroll
+            for (int n1 = 0; n1 < P; ++n1) o[n1] = T[(g + G * u) * (P + 1) + n1];
+            reg_fft<P, INV>(o);
+#pragma unroll
+            for (int k1 = 0; k1 < P; ++k1) out[u * P + k1] = o[k1];
+        }
     }
     __syncwarp();
 }
