@@ -470,12 +470,16 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
         __syncthreads();                          // the batch's phasors are visible to all
     }
     // the result, from the table (FP64 conversions in the chain above would
-    // queue at the SM's slow FP64 unit)
-    for (int e = (int)rank * TH + tid; e < p.hb_rows * p.box_cols; e += (int)cl * TH) {
-        const int ky = e / p.box_cols, kx = e - ky * p.box_cols - K, q = kx * kx + ky * ky;
-        if (q < 2 || q > p.r2i) continue;
-        const T2 t = zget(zs, (ky * zp + kx) * ZB);
-        zo[ky * p.box_pitch + kx + K] = make_double2((double)t.x, (double)t.y);
+    // queue at the SM's slow FP64 unit); zero outside the cutoff
+    for (int e = (int)rank * TH + tid; e < (int)hb; e += (int)cl * TH) {
+        const int ky = e / p.box_pitch, kx = e - ky * p.box_pitch - K, q = kx * kx + ky * ky;
+        if (q < 2) continue;
+        double2 v = make_double2(0.0, 0.0);
+        if (q <= p.r2i) {
+            const T2 t = zget(zs, (ky * zp + kx) * ZB);
+            v = make_double2((double)t.x, (double)t.y);
+        }
+        zo[e] = v;
     }
 }
 

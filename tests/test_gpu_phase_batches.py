@@ -80,3 +80,23 @@ def test_phasors_do_not_depend_on_the_cluster(torch, phase):
     for k, z in got.items():
         assert np.array_equal(z[:k], got[n][:k]), k
         assert not z[k:].any(), k
+
+
+@pytest.mark.parametrize("N,R,prec", [(64, 8, 0), (128, 5, 1), (256, 3, 2)])
+def test_phasors_are_written_whole(torch, N, R, prec):
+    """Every value of z is written, zero outside the cutoff, whatever the workspace held."""
+    from paper_1701_00581_gb300 import Channel, Plan
+    plan = Plan(Channel(W=N, H=N, N=N, R=R, phase_prec=prec, max_frames=2))
+    ws, lay = plan.workspace(2, 1)
+    ws.view(torch.uint8).fill_(0xff)
+    frames = torch.from_numpy(np.random.default_rng(N).random((2, N, N), dtype=np.float32) + 1).cuda()
+    plan.stage_spectra(frames, 2, 0, 1, ws, lay)
+    plan.stage_stats(2, 1, ws, lay)
+    plan.stage_bispectrum(2, 1, ws, lay)
+    plan.stage_phase(1, ws, lay)
+    z = plan.views(ws, lay, 2, 1)["z"][0].cpu().numpy()
+    K = plan.info["K"]
+    ky, kx = np.mgrid[0:z.shape[0], -K:z.shape[1] - K]
+    inside = kx ** 2 + ky ** 2 <= (0.2885 * N) ** 2
+    assert np.isfinite(z.view(np.float64)).all()
+    assert (z[~inside] == 0).all() and (np.abs(np.abs(z[inside]) - 1) <= 1e-6).all()
