@@ -39,7 +39,7 @@
 // zero-filled frames, which add nothing to the sums.  Accumulators are
 // written once per burst.
 //
-// 304 subfields of 256^2, R = 24, 100 frames: 102.0 -> 88 ms; 225 of 128^2,
+// 304 subfields of 256^2, R = 24, 100 frames: 102.0 -> 89.4 ms; 225 of 128^2,
 // R = 16: 11.5 -> 8.7 ms; one of 64^2, R = 8: 47 -> 42 us; 15 of 256^2 with FP16
 // spectra 6.2 -> 5.4 ms, with compensated sums too 9.0 -> 8.8 ms.
 #include "sm_bispec_tile.cuh"
