@@ -174,8 +174,8 @@ __device__ __forceinline__ void chunk_copy(const PlanDev& p, int c, int rows, in
 // One task (blockIdx-free) of subfield slot `sl`: B of spec[sl] at the task's
 // pairs into B[sl]; S is the CTA's staging area, staging_float2<PREC, KAHAN>() float2
 // of 16-byte aligned shared memory (2 FB BUF for FP32 spectra, 3 FB BUF for
-// half precision).  Runs on 128 threads; uses __syncthreads, so the whole CTA
-// must call it.  VCH: V starts at an even box column.  KAHAN: blocked
+// half precision).  Runs on 128 threads and synchronises them (barriers 0 and
+// 1), so the whole CTA must call it.  VCH: V starts at an even box column.  KAHAN: blocked
 // compensated sums -- each block of two stages (2 FB frames) is summed plainly
 // into a partial, which is then added to the running sum with Kahan
 // compensation; partial, sum and correction fill the registers of 4 columns
@@ -273,9 +273,14 @@ __device__ __forceinline__ void bispec_tile(const PlanDev& p, const void* __rest
             }
     };
     // Stage st ready in shared memory, the next on its way; the frames' buffers.
+    // A CTA's warps come here from different code, each from the loop made for
+    // its columns, which __syncthreads() does not allow; a barrier named by its
+    // number, on which every warp arrives for its 32 threads, does.  Every
+    // branch below calls this nst times.
     auto next_stage = [&](int st) -> const float2* {
-        asm volatile("cp.async.wait_group 0;");
-        __syncthreads();              // stage st visible to all; stage st-1 fully consumed
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        // stage st visible to all; stage st-1 fully consumed
+        asm volatile("bar.sync 1, %0;" :: "n"(THREADS) : "memory");
         if constexpr (RAW) {
             issue(st + 2);
             if (st + 1 < nst) convert(st + 1);
@@ -367,6 +372,7 @@ __device__ __forceinline__ void bispec_tile(const PlanDev& p, const void* __rest
     };
 #pragma unroll
     for (int pass = 0; pass < NP; ++pass) {
+        __syncwarp();                              // a warp's idle lanes leave run() before the others
         if (pass > 0) __syncthreads();             // the previous pass is done with the ring
         issue(0);
         if constexpr (RAW) {
