@@ -35,11 +35,11 @@
 //
 // Every sum runs in a fixed order (per lane over a unit's rows, a butterfly
 // over the lanes; a point's units and late terms over the lanes, a
-// butterfly), so the result does not depend on scheduling, on the CTA size or
-// on the cluster.  Arithmetic is FP32 by default
-// (GB300's FP64 unit is shared by the SM's warps and a small fraction of its
-// FP32 rate), or FP64 or float-float when the channel asks for it; the known
-// phasors live in shared memory in that type and the result is stored as FP64.
+// butterfly), so the result does not depend on scheduling or on the cluster.
+// Arithmetic is FP32 by default (GB300's FP64 unit is shared by the SM's warps
+// and a small fraction of its FP32 rate), or FP64 or float-float when the
+// channel asks for it; the known phasors live in shared memory in that type
+// and the result is stored as FP64.
 #include <type_traits>
 
 #include "sm_internal.h"
@@ -49,7 +49,7 @@ namespace {
 using smi::PlanDev;
 using smi::TILE_PAIRS;
 
-constexpr int PH_WARPS = 16;           // warps of the largest CTA
+constexpr int PH_WARPS = 16, TH = 32 * PH_WARPS;   // warps and threads of a CTA
 constexpr int PH_STEPS = 8;            // steps of 4 tile rows whose B loads are in flight together
 constexpr int PH_LATE_WARPS = 8;       // warps that walk the rings (a ring has 4 to 6 points on average)
 
@@ -152,7 +152,7 @@ __host__ __device__ inline PhaseLayout phase_layout(int hb_rows, int zpitch, int
     l.liv = l.lb + (size_t)max_late * sizeof(float2);
     l.rs = l.liv + (size_t)max_late * sizeof(int);
     l.ent = (l.rs + (size_t)(max_points + 1) * sizeof(int) + 15) & ~(size_t)15;
-    l.bytes = l.ent + (size_t)PH_WARPS * 32 * sizeof(int2);
+    l.bytes = l.ent + (size_t)TH * sizeof(int2);
     return l;
 }
 
@@ -210,11 +210,10 @@ template <typename T2> __device__ __forceinline__ void store_cluster(T2* at, uns
 }
 
 // WEIGHT: the term weighting (SM_W_*).
-template <typename T, int TH, int WEIGHT>
-__global__ void __launch_bounds__(TH, TH == 512 ? (sizeof(T) == 4 ? 2 : 1) : 4)
+template <typename T, int WEIGHT>
+__global__ void __launch_bounds__(TH, sizeof(T) == 4 ? 2 : 1)
 k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, const float* __restrict__ P,
         double2* __restrict__ z) {
-    constexpr int NW = TH / 32;
     using T2 = typename Cx<T>::T2;
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, zp = p.zpitch;
@@ -291,7 +290,7 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
     // where a whole tile kept 53 %.  The lanes load the entries, one unit
     // ahead, and read them back from shared memory; a unit's record comes two
     // units ahead, those of the batch's first units during the batch before.
-    const int l8 = lane & 7, stride = (int)cl * NW, first = (int)rank * NW + warp;
+    const int l8 = lane & 7, stride = (int)cl * PH_WARPS, first = (int)rank * PH_WARPS + warp;
     int2 unit0 = make_int2(0, 0), unit1 = make_int2(0, 0), mine = make_int2(0, 0);
     auto load_unit = [&](int u, int u1) { return u < u1 ? __ldg(p.units + u) : make_int2(0, 0); };
     auto load_entries = [&](int2 unit) {                   // a unit: first entry, entries | point << 6
@@ -339,9 +338,8 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
 
     // What a batch needs in shared memory before its sums: records, ring
     // starts and late terms.  The warps that do not walk the rings load the
-    // next batch's into registers while the others do (256 threads: all walk,
-    // and the loads follow).
-    constexpr int PF_THREADS = NW > PH_LATE_WARPS ? (NW - PH_LATE_WARPS) * 32 : TH;
+    // next batch's into registers while the others do.
+    constexpr int PF_THREADS = (PH_WARPS - PH_LATE_WARPS) * 32;
     constexpr int PF = smi::PHASE_LATE / 256;               // late terms per loading thread
     static_assert(PF_THREADS >= 256 && 2 * smi::PHASE_BATCH_MAX <= PF_THREADS, "one record, PF late terms per thread");
     struct Ahead {
@@ -406,8 +404,9 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
         if (cl > 1) cluster_sync();
         else __syncthreads();
         mine = load_entries(unit0);
-        if (NW == PH_LATE_WARPS || warp >= PH_LATE_WARPS) load_ahead(ahead, bt + 1);
-        if (warp < PH_LATE_WARPS) {
+        if (warp >= PH_LATE_WARPS) {
+            load_ahead(ahead, bt + 1);
+        } else {
             // Points go round the walking warps in order, so that the few
             // warps with a point in one ring are mostly not those of the
             // next: a warp reads its next point's record, early sums and
@@ -497,18 +496,18 @@ namespace {
 // CTAs per subfield: as many as keep the whole grid resident (two CTAs per SM
 // when their shared memory allows it) and a unit of the largest batch for
 // every warp, up to a portable cluster of 8.
-template <typename T, int TH, int WEIGHT>
+template <typename T, int WEIGHT>
 cudaError_t phase_go(const smi::PlanDev& p, int nsub, const float2* B, const float2* M, const float* P, double2* z,
                      size_t sm, cudaStream_t st) {
-    auto* const kern = k_phase<T, TH, WEIGHT>;
+    auto* const kern = k_phase<T, WEIGHT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     int dev = 0, sms = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int slots = sms * (TH == 512 && sizeof(T) == 4 && sm <= 113 * 1024 ? 2 : 1);
+    const int slots = sms * (sizeof(T) == 4 && sm <= 113 * 1024 ? 2 : 1);
     int cl = 1;
-    while (TH == 512 && cl < 8 && nsub * 2 * cl <= slots && 2 * cl * PH_WARPS <= p.max_batch_units) cl *= 2;
+    while (cl < 8 && nsub * 2 * cl <= slots && 2 * cl * PH_WARPS <= p.max_batch_units) cl *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nsub * cl);
     cfg.blockDim = dim3(TH);
@@ -523,24 +522,23 @@ cudaError_t phase_go(const smi::PlanDev& p, int nsub, const float2* B, const flo
     return cudaLaunchKernelEx(&cfg, kern, p, B, M, P, z);
 }
 
-template <typename T, int TH>
+template <typename T>
 cudaError_t phase_weighted(const smi::PlanDev& p, int nsub, const float2* B, const float2* M, const float* P, double2* z,
                            size_t sm, cudaStream_t st) {
-    if (p.weight == SM_W_UNIT) return phase_go<T, TH, SM_W_UNIT>(p, nsub, B, M, P, z, sm, st);
-    if (p.weight == SM_W_SNR) return phase_go<T, TH, SM_W_SNR>(p, nsub, B, M, P, z, sm, st);
-    return phase_go<T, TH, SM_W_BISPEC>(p, nsub, B, M, P, z, sm, st);
+    if (p.weight == SM_W_UNIT) return phase_go<T, SM_W_UNIT>(p, nsub, B, M, P, z, sm, st);
+    if (p.weight == SM_W_SNR) return phase_go<T, SM_W_SNR>(p, nsub, B, M, P, z, sm, st);
+    return phase_go<T, SM_W_BISPEC>(p, nsub, B, M, P, z, sm, st);
 }
 
 }  // namespace
 
 cudaError_t launch_phase(const smi::PlanDev& p, int nsub, const float2* B, const float2* M, const float* P,
-                         double2* z, cudaStream_t st, int threads) {
+                         double2* z, cudaStream_t st) {
     const size_t sm = phase_smem_bytes(p.hb_rows, p.zpitch, p.max_batch_points, p.max_batch_units, p.max_batch_late,
                                        p.phase_prec);
-    if (p.phase_prec == SM_PHASE_FP64) return phase_weighted<double, 512>(p, nsub, B, M, P, z, sm, st);
-    if (p.phase_prec == SM_PHASE_FF) return phase_weighted<ff, 512>(p, nsub, B, M, P, z, sm, st);
-    if (threads == 256) return phase_weighted<float, 256>(p, nsub, B, M, P, z, sm, st);
-    return phase_weighted<float, 512>(p, nsub, B, M, P, z, sm, st);
+    if (p.phase_prec == SM_PHASE_FP64) return phase_weighted<double>(p, nsub, B, M, P, z, sm, st);
+    if (p.phase_prec == SM_PHASE_FF) return phase_weighted<ff>(p, nsub, B, M, P, z, sm, st);
+    return phase_weighted<float>(p, nsub, B, M, P, z, sm, st);
 }
 
 }  // namespace smk

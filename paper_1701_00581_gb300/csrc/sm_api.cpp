@@ -341,25 +341,9 @@ int reconstruct_check(const sm_plan* plan, int F, const double* stf, int nsub_ch
 
 // Run a schedule; with `marks`, marks[i] is recorded on the stream before
 // call i and marks[calls.size()] after the last (timing of each call).
-// The phase stage with the recursion kernel at `threads` threads a CTA (512:
-// the stage path; 256: small enough to share an SM with three bispectrum
-// CTAs; bitwise the same phasors).
-int stage_phase_threads(const sm_plan* plan, int nsub, void* ws, const sm_workspace_layout* lay, void* stream,
-                        int threads) {
-    if (threads == 512 || plan->dev.phase_prec != SM_PHASE_FP32) return sm_stage_phase(plan, nsub, ws, lay, stream);
-    DeviceGuard g(plan->device);
-    int rc = ret(smk::launch_phase(plan->dev, nsub, at<float2>(ws, lay->B), at<float2>(ws, lay->M),
-                                   at<float>(ws, lay->P), at<double2>(ws, lay->z), (cudaStream_t)stream, threads),
-                 "phase kernel");
-    if (rc || plan->dev.phase_iters == 0) return rc;
-    return ret(smk::launch_refine(plan->dev, nsub, at<float2>(ws, lay->B), at<float>(ws, lay->P),
-                                  at<double2>(ws, lay->z), at<float2>(ws, lay->refine), (cudaStream_t)stream),
-               "least-squares phase sweeps");
-}
-
 int run_schedule(const sm_plan* plan, const std::vector<StageCall>& calls, const void* frames, int frame_type,
                  int F, const double* stf, void* ws, const sm_workspace_layout* lay, float* out, uint8_t* valid,
-                 void* stream, const std::vector<cudaEvent_t>* marks, int phase_threads = 512) {
+                 void* stream, const std::vector<cudaEvent_t>* marks) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     auto mark = [&](size_t i) -> int {
         if (!marks) return SM_OK;
@@ -376,7 +360,7 @@ int run_schedule(const sm_plan* plan, const std::vector<StageCall>& calls, const
         case ST_SEEING_STF: rc = sm_stage_seeing_stf(plan, ws, lay, stream); break;
         case ST_AMPLITUDE: rc = sm_stage_amplitude(plan, c.ns, stf, ws, lay, stream); break;
         case ST_BISPECTRUM: rc = sm_stage_bispectrum(plan, F, c.ns, ws, lay, stream); break;
-        case ST_PHASE: rc = stage_phase_threads(plan, c.ns, ws, lay, stream, phase_threads); break;
+        case ST_PHASE: rc = sm_stage_phase(plan, c.ns, ws, lay, stream); break;
         case ST_INVERSE: rc = sm_stage_inverse(plan, F, c.s0, c.ns, ws, lay, stream); break;
         case ST_MOSAIC: rc = sm_stage_mosaic(plan, ws, lay, out, valid, stream); break;
         }
@@ -601,8 +585,10 @@ namespace {
 // STF mode (given, or estimated on the device when d_stf is NULL) are part
 // of the captured kernels, so they join the key through the F slot.
 // part 0: the whole schedule; pipelined: 1 the stages before the bispectrum,
-// 3 the bispectrum, 2 the back half (phase .. mosaic, with the 256-thread
-// phase kernel); wsi: the pipelined workspace the burst uses.
+// 3 the bispectrum, 2 the back half (phase .. mosaic); wsi: the pipelined
+// workspace the burst uses.  The back half runs the recursion as the stage path
+// does, as a cluster of CTAs per subfield when there are few: 15 subfields of
+// 256^2 served pipelined 177 bursts/s, against 116 with one small CTA each.
 int launch_burst(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, const double* d_stf,
                  void* ws, sm_workspace_layout& lay, cudaStream_t st, int part = 0, int wsi = 0) {
     const auto key = std::make_tuple(b->channel, b->F * 4 + (d_stf ? 0 : 2) + (b->frame_type == SM_F32 ? 1 : 0),
@@ -643,7 +629,7 @@ int launch_burst(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, 
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaStreamBeginCapture"); }
         rc = run_schedule(plan, calls, d_frames, b->frame_type, b->F, stf_used, ws, &lay, j.d_out, j.d_valid, st,
-                          &ng.marks, part == 2 ? 256 : 512);
+                          &ng.marks);
         if (rc == SM_OK && j.d_seeing_io && (part == 0 || part == 2))
             rc = ret(cudaMemcpyAsync(j.d_seeing_io, j.d_seeing, sizeof(double), cudaMemcpyDeviceToDevice, st),
                      "cudaMemcpyAsync(seeing)");

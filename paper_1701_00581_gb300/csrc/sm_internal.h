@@ -178,7 +178,7 @@ cudaError_t launch_bispectrum(const smi::PlanDev& p, const void* spec, int F, in
 cudaError_t launch_refine(const smi::PlanDev& p, int nsub, const float2* B, const float* P, double2* z,
                           float2* partials, cudaStream_t st);
 cudaError_t launch_phase(const smi::PlanDev& p, int nsub, const float2* B, const float2* M, const float* P,
-                         double2* z, cudaStream_t st, int threads = 512);
+                         double2* z, cudaStream_t st);
 cudaError_t launch_inverse(const smi::PlanDev& p, int F, int sub0, int nsub, const float* A,
                            const double2* z, const float* flux, const float* mu, float* rec,
                            cudaStream_t st);

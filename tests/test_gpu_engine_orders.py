@@ -1,0 +1,44 @@
+"""The pipelined kernel order beside the submission order, on a burst of few subfields."""
+from __future__ import annotations
+
+import time
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def test_pipelined_order_is_not_slower():
+    """Both orders run the same kernels; the pipelined one puts a burst's recursion beside the next burst's
+    bispectrum, so it has to serve no fewer bursts, less a tenth for the order's own overheads.  The best of three
+    runs of each counts."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("no CUDA device")
+    from paper_1701_00581_gb300 import Channel, Engine
+    W, H, F, n = 768, 512, 100, 24
+    rng = np.random.default_rng(5)
+    frames = torch.from_numpy(rng.integers(900, 3000, (F, H, W)).astype(np.uint16)).pin_memory()
+    d = rng.uniform(5.0, 10.0, F)
+    outs = [torch.empty((H, W), dtype=torch.float32).pin_memory() for _ in range(3)]
+
+    def serve(eng, k):
+        flying = []
+        t0 = time.perf_counter()
+        for i in range(k):
+            if len(flying) == 3:
+                eng.poll(flying.pop(0), -1)
+            flying.append(eng.submit(0, frames.numpy(), outs[i % 3].numpy(), None, d_over_r0=d))
+        for t in flying:
+            eng.poll(t, -1)
+        return k / (time.perf_counter() - t0)
+
+    rate = {}
+    for mode in (0, 2):
+        eng = Engine([Channel(W=W, H=H, N=256, R=24, max_frames=F)], hbm_budget_bytes=40 << 30, max_inflight=3,
+                     overlap_kernels=mode)
+        serve(eng, 6)
+        rate[mode] = max(serve(eng, n) for _ in range(3))
+        eng.close()
+    assert rate[2] >= 0.9 * rate[0], rate
