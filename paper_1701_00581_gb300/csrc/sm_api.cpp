@@ -580,69 +580,78 @@ void finish_job(sm_handle* h, Job& j) {
 
 namespace {
 
-// Launch one burst's stage sequence on its slot stream through a cached
-// CUDA graph (captured on first use of the key).  The frame type and the
-// STF mode (given, or estimated on the device when d_stf is NULL) are part
-// of the captured kernels, so they join the key through the F slot.
+// The CUDA graph of a burst's stage sequence, captured on first use of its key
+// (and uploaded then).  The frame type and the STF mode (given, or estimated
+// on the device when d_stf is NULL) are part of the captured kernels, so they
+// join the key through the F slot.
 // part 0: the whole schedule; pipelined: 1 the stages before the bispectrum,
 // 3 the bispectrum, 2 the back half (phase .. mosaic); wsi: the pipelined
 // workspace the burst uses.  The back half runs the recursion as the stage path
 // does, as a cluster of CTAs per subfield when there are few: 15 subfields of
 // 256^2 served pipelined 177 bursts/s, against 116 with one small CTA each.
-int launch_burst(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, const double* d_stf,
-                 void* ws, sm_workspace_layout& lay, cudaStream_t st, int part = 0, int wsi = 0) {
+int burst_graph(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, const double* d_stf, void* ws,
+                sm_workspace_layout& lay, cudaStream_t st, int part, int wsi, sm_handle::Graph** out) {
     const auto key = std::make_tuple(b->channel, b->F * 4 + (d_stf ? 0 : 2) + (b->frame_type == SM_F32 ? 1 : 0),
                                      j.off, j.slot * 16 + part * 4 + wsi);
-    sm_handle::Graph* g = nullptr;
     {
         std::lock_guard<std::mutex> lk(h->mu);
         auto it = h->graphs.find(key);
-        if (it != h->graphs.end()) g = &it->second;
+        if (it != h->graphs.end()) { *out = &it->second; return SM_OK; }
     }
-    if (!g) {
-        const sm_plan* plan = h->plans[b->channel];
-        const double* stf_used = nullptr;
-        int rc = reconstruct_check(plan, b->F, d_stf, h->chunk[b->channel], ws, &lay, &stf_used);
-        if (rc) return rc;
-        std::vector<StageCall> calls = burst_schedule(plan, d_stf == nullptr, h->chunk[b->channel]);
-        if (part) {
-            // the schedule of an unchunked burst, cut before the bispectrum
-            // and before the phase
-            size_t cb = 0, cp = 0;
-            while (cb < calls.size() && calls[cb].stage != ST_BISPECTRUM) ++cb;
-            while (cp < calls.size() && calls[cp].stage != ST_PHASE) ++cp;
-            if (part == 1) calls = std::vector<StageCall>(calls.begin(), calls.begin() + cb);
-            else if (part == 3) calls = std::vector<StageCall>(calls.begin() + cb, calls.begin() + cp);
-            else calls = std::vector<StageCall>(calls.begin() + cp, calls.end());
-        }
-        sm_handle::Graph ng;
-        for (const StageCall& c : calls) ng.stage.push_back(reported_stage(c.stage));
-        ng.marks.assign(calls.size() + 1, nullptr);
-        auto drop = [&](cudaGraph_t graph) {
-            if (graph) cudaGraphDestroy(graph);
-            for (auto ev : ng.marks) if (ev) cudaEventDestroy(ev);
-        };
-        for (auto& ev : ng.marks) {
-            cudaError_t e = cudaEventCreate(&ev);
-            if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaEventCreate"); }
-        }
-        cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaStreamBeginCapture"); }
-        rc = run_schedule(plan, calls, d_frames, b->frame_type, b->F, stf_used, ws, &lay, j.d_out, j.d_valid, st,
-                          &ng.marks);
-        if (rc == SM_OK && j.d_seeing_io && (part == 0 || part == 2))
-            rc = ret(cudaMemcpyAsync(j.d_seeing_io, j.d_seeing, sizeof(double), cudaMemcpyDeviceToDevice, st),
-                     "cudaMemcpyAsync(seeing)");
-        cudaGraph_t graph = nullptr;
-        e = cudaStreamEndCapture(st, &graph);
-        if (rc != SM_OK) { drop(graph); return rc; }
-        if (e != cudaSuccess) { drop(graph); return cuda_fail(e, "cudaStreamEndCapture"); }
-        e = cudaGraphInstantiate(&ng.exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaGraphInstantiate"); }
-        std::lock_guard<std::mutex> lk(h->mu);
-        g = &(h->graphs[key] = std::move(ng));
+    const sm_plan* plan = h->plans[b->channel];
+    const double* stf_used = nullptr;
+    int rc = reconstruct_check(plan, b->F, d_stf, h->chunk[b->channel], ws, &lay, &stf_used);
+    if (rc) return rc;
+    std::vector<StageCall> calls = burst_schedule(plan, d_stf == nullptr, h->chunk[b->channel]);
+    if (part) {
+        // the schedule of an unchunked burst, cut before the bispectrum
+        // and before the phase
+        size_t cb = 0, cp = 0;
+        while (cb < calls.size() && calls[cb].stage != ST_BISPECTRUM) ++cb;
+        while (cp < calls.size() && calls[cp].stage != ST_PHASE) ++cp;
+        if (part == 1) calls = std::vector<StageCall>(calls.begin(), calls.begin() + cb);
+        else if (part == 3) calls = std::vector<StageCall>(calls.begin() + cb, calls.begin() + cp);
+        else calls = std::vector<StageCall>(calls.begin() + cp, calls.end());
     }
+    sm_handle::Graph ng;
+    for (const StageCall& c : calls) ng.stage.push_back(reported_stage(c.stage));
+    ng.marks.assign(calls.size() + 1, nullptr);
+    auto drop = [&](cudaGraph_t graph) {
+        if (graph) cudaGraphDestroy(graph);
+        for (auto ev : ng.marks) if (ev) cudaEventDestroy(ev);
+    };
+    for (auto& ev : ng.marks) {
+        cudaError_t e = cudaEventCreate(&ev);
+        if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaEventCreate"); }
+    }
+    cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaStreamBeginCapture"); }
+    rc = run_schedule(plan, calls, d_frames, b->frame_type, b->F, stf_used, ws, &lay, j.d_out, j.d_valid, st,
+                      &ng.marks);
+    if (rc == SM_OK && j.d_seeing_io && (part == 0 || part == 2))
+        rc = ret(cudaMemcpyAsync(j.d_seeing_io, j.d_seeing, sizeof(double), cudaMemcpyDeviceToDevice, st),
+                 "cudaMemcpyAsync(seeing)");
+    cudaGraph_t graph = nullptr;
+    e = cudaStreamEndCapture(st, &graph);
+    if (rc != SM_OK) { drop(graph); return rc; }
+    if (e != cudaSuccess) { drop(graph); return cuda_fail(e, "cudaStreamEndCapture"); }
+    e = cudaGraphInstantiate(&ng.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) { drop(nullptr); return cuda_fail(e, "cudaGraphInstantiate"); }
+    e = cudaGraphUpload(ng.exec, st);
+    if (e != cudaSuccess) { cudaGraphExecDestroy(ng.exec); drop(nullptr); return cuda_fail(e, "cudaGraphUpload"); }
+    std::lock_guard<std::mutex> lk(h->mu);
+    *out = &(h->graphs[key] = std::move(ng));
+    return SM_OK;
+}
+
+// Launch a part of a burst (burst_graph) on stream st.  The burst's device time
+// starts here with its first part: capturing the graph is not part of it.
+int launch_burst(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, const double* d_stf,
+                 void* ws, sm_workspace_layout& lay, cudaStream_t st, int part = 0, int wsi = 0) {
+    sm_handle::Graph* g = nullptr;
+    int rc = burst_graph(h, b, j, d_frames, d_stf, ws, lay, st, part, wsi, &g);
+    if (rc) return rc;
     if (part == 2) {
         j.marks2 = &g->marks;
         j.mark_stage2 = &g->stage;
@@ -652,6 +661,8 @@ int launch_burst(sm_handle* h, const sm_burst* b, Job& j, const void* d_frames, 
     } else {
         j.marks = &g->marks;
         j.mark_stage = &g->stage;
+        rc = ret(cudaEventRecord(j.ev_start, st), "cudaEventRecord");
+        if (rc) return rc;
     }
     return ret(cudaGraphLaunch(g->exec, st), "cudaGraphLaunch");
 }
@@ -967,14 +978,18 @@ extern "C" int sm_submit_burst(sm_handle* h, const sm_burst* b, uint64_t* ticket
         void* wsw = h->ws2[w];
         if (h->front_recorded) e = cudaStreamWaitEvent(st, h->ev_front, 0);
         if (e == cudaSuccess && h->free_recorded[w]) e = cudaStreamWaitEvent(st, h->ev_free[w], 0);
-        if (e == cudaSuccess) e = cudaEventRecord(j.ev_start, st);
         if (e == cudaSuccess && !j.ev_mid) e = cudaEventCreateWithFlags(&j.ev_mid, cudaEventDisableTiming);
         if (e == cudaSuccess && !j.ev_bis) e = cudaEventCreateWithFlags(&j.ev_bis, cudaEventDisableTiming);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "ordering burst");
         } else {
             if (j.d_seeing) j.d_seeing = at<double>(wsw, lay.seeing) + h->plans[b->channel]->dev.n_cubes;
-            rc = launch_burst(h, b, j, d_frames, est ? nullptr : d_stf, wsw, lay, st, 1, w);
+            // every part captured before the first is launched
+            sm_handle::Graph* g = nullptr;
+            rc = burst_graph(h, b, j, d_frames, est ? nullptr : d_stf, wsw, lay, st, 1, w, &g);
+            if (rc == SM_OK) rc = burst_graph(h, b, j, d_frames, est ? nullptr : d_stf, wsw, lay, lo, 3, w, &g);
+            if (rc == SM_OK) rc = burst_graph(h, b, j, d_frames, est ? nullptr : d_stf, wsw, lay, ph, 2, w, &g);
+            if (rc == SM_OK) rc = launch_burst(h, b, j, d_frames, est ? nullptr : d_stf, wsw, lay, st, 1, w);
         }
         if (rc == SM_OK) {
             e = cudaEventRecord(j.ev_mid, st);
@@ -988,7 +1003,6 @@ extern "C" int sm_submit_burst(sm_handle* h, const sm_burst* b, uint64_t* ticket
             h->front_recorded = e == cudaSuccess;
             if (e != cudaSuccess) rc = cuda_fail(e, "ordering burst");
         }
-        (void)ph;
         // the previous burst's back half now goes after this burst's early
         // stages; this burst's waits for the next burst (or its poll)
         if (rc == SM_OK && h->pending_back) {
@@ -1017,11 +1031,10 @@ extern "C" int sm_submit_burst(sm_handle* h, const sm_burst* b, uint64_t* ticket
     } else {
         std::lock_guard<std::mutex> lk(h->launch_mu);
         if (!h->cfg.overlap_kernels && h->ordered) {
-            // queue behind the previous burst's kernels; ev_start is taken
-            // again after the wait so that gpu_ms counts this burst's own
+            // queue behind the previous burst's kernels; launch_burst takes
+            // ev_start after the wait, so that gpu_ms counts this burst's own
             // kernels only
             e = cudaStreamWaitEvent(st, h->order, 0);
-            if (e == cudaSuccess) e = cudaEventRecord(j.ev_start, st);
         }
         if (e != cudaSuccess) rc = cuda_fail(e, "ordering burst");
         else rc = launch_burst(h, b, j, d_frames, est ? nullptr : d_stf, ws, lay, st);
@@ -1154,7 +1167,6 @@ extern "C" int sm_submit_batch(sm_handle* h, int n, const sm_burst* bs, uint64_t
         cudaStream_t st = h->streams[js[0].slot];
         if (h->ordered) e = cudaStreamWaitEvent(st, h->order, 0);
         for (int i = 1; i < n && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(st, js[i].ev_start, 0);
-        for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaEventRecord(js[i].ev_start, st);
         if (e != cudaSuccess) rc = cuda_fail(e, "ordering batch");
         sm_batch* bt = nullptr;
         if (rc == SM_OK) {
@@ -1192,6 +1204,8 @@ extern "C" int sm_submit_batch(sm_handle* h, int n, const sm_burst* bs, uint64_t
                     if (rc == SM_OK && e != cudaSuccess) rc = cuda_fail(e, "cudaStreamEndCapture");
                     if (rc == SM_OK) {
                         e = cudaGraphInstantiate(&ng.exec, graph, 0);
+                        if (e == cudaSuccess && (e = cudaGraphUpload(ng.exec, st)) != cudaSuccess)
+                            cudaGraphExecDestroy(ng.exec);
                         if (e != cudaSuccess) rc = cuda_fail(e, "cudaGraphInstantiate");
                     }
                     if (graph) cudaGraphDestroy(graph);
@@ -1201,6 +1215,8 @@ extern "C" int sm_submit_batch(sm_handle* h, int n, const sm_burst* bs, uint64_t
                     gr = &(h->bgraphs[gk] = std::move(ng));
                 }
             }
+            // the bursts' device time starts here, with the graph at hand
+            for (int i = 0; i < n && rc == SM_OK; ++i) rc = ret(cudaEventRecord(js[i].ev_start, st), "cudaEventRecord");
             if (rc == SM_OK) rc = ret(cudaGraphLaunch(gr->exec, st), "cudaGraphLaunch");
         }
         if (rc == SM_OK) {

@@ -42,3 +42,24 @@ def test_pipelined_order_is_not_slower():
         rate[mode] = max(serve(eng, n) for _ in range(3))
         eng.close()
     assert rate[2] >= 0.9 * rate[0], rate
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_device_time_of_an_engines_first_burst(mode):
+    """gpu_ms counts the burst's device time, not the host's capture of its graph: the stages account for half of it
+    at least, from an engine's first burst on (ten engines, so that one lucky first burst does not pass for all)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("no CUDA device")
+    from paper_1701_00581_gb300 import Engine
+    from synth import burst as S
+    from tests import _cases as CS
+    ch = CS.gpu_channel("ragged")
+    b = S.make_burst(CS.RAGGED["spec"], channel=11, burst=0)
+    out = np.zeros((ch.H, ch.W), np.float32)
+    for _ in range(10):
+        eng = Engine([ch], hbm_budget_bytes=1 << 30, max_inflight=2, overlap_kernels=mode)
+        for _ in range(2):
+            st, res = eng.poll(eng.submit(0, b["frames"], out, d_over_r0=b["d_over_r0"]), -1)
+            assert st == 0 and sum(res["stage_ms"].values()) >= 0.5 * res["gpu_ms"]
+        eng.close()
