@@ -206,7 +206,8 @@ int sm_stage_calibrate(const sm_plan* plan, const void* raw, int frame_type, int
  * ref_window: device float [G][G] scratch; cc: device double
  * [F][2S+1][2S+1] receives C; shifts: device int [F][2] receives (sx, sy).
  * SM_EINVAL unless 0 <= S <= 31 and the window moved by +-S fits the frame
- * ((W-G)/2 >= S, (W-G)/2 + G + S <= W, and likewise in y).                */
+ * ((W-G)/2 >= S, (W-G)/2 + G + S <= W, and likewise in y), G + S <= 29056
+ * and F <= 65535.                                                          */
 int sm_stage_track(const sm_plan* plan, const void* frames, int frame_type, int F, int ref, int G, int S,
                    float* ref_window, double* cc, int* shifts, void* stream);
 

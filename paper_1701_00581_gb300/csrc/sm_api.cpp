@@ -128,6 +128,10 @@ extern "C" int sm_stage_track(const sm_plan* plan, const void* frames, int frame
     if (S < 0 || S > smk::track_max_search() || G < 1 || x0 < S || y0 < S || x0 + G + S > W || y0 + G + S > H) {
         set_error("tracking window plus search range does not fit the frame (or S > 31)"); return SM_EINVAL;
     }
+    // the kernels index the window's samples with int
+    if (2 * ((size_t)G + S) * sizeof(float) > 227 * 1024 || F > 65535) {
+        set_error("tracking needs G + S <= 29056 and F <= 65535"); return SM_EINVAL;
+    }
     DeviceGuard g(plan->device);
     return ret(smk::launch_track(plan->dev, frames, frame_type, F, ref, G, S, ref_window, cc, shifts,
                                  (cudaStream_t)stream),
