@@ -128,10 +128,12 @@ cudaError_t launch_calibrate(const smi::PlanDev& p, const void* raw, int frame_t
 // a thread owns 12 neighbouring shifts sx of one sy and slides a register
 // window along the row, so 4 samples cost two 16-byte shared loads and 48
 // FMAs (bound by FP32 FMA issue: 100 frames, G = 256, S = 16 in 0.52 ms, with
-// the pick; one thread per shift and row by row staging took 3.3 + 0.53 ms).  Products are summed in FP32 over 32-sample chunks; the chunks are
-// summed as float-float pairs (48 bits, on the FP32 pipe: adding each chunk in
+// the pick; one thread per shift and row by row staging took 3.3 + 0.53 ms).
+// Products are summed in FP32 over 32-sample chunks; the chunks are summed as
+// float-float pairs (48 bits, on the FP32 pipe: adding each chunk in
 // FP64 would alone take 0.4 ms for 100 frames of a 256^2 window and S = 16 on
-// GB300's FP64 units), and threads and CTAs in FP64.  The cluster's first CTA
+// GB300's FP64 units), or in FP64 where a pair's sum is not finite, and threads
+// and CTAs in FP64.  The cluster's first CTA
 // writes the surface and picks the first maximum.  k_shift: a warp per row
 // (100 float frames of 2560 x 2160, 4.4 GB: 1.78 -> 0.67 ms, 6.7 TB/s).
 namespace {
@@ -221,6 +223,24 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float p) {
     hi = s;
 }
 
+// One shift's products over a thread's share of the window rows [ya, yb) -- of
+// every RB rows those share, share + rs, ... -- from the frame at (x0, y0), as
+// the kernel below forms them, the chunks summed in FP64.
+template <typename In>
+__device__ __noinline__ double row_share_fp64(const In* a, int W, int x0, int y0, int G, int ya, int yb, int share, int rs,
+                                              const float* rw) {
+    double t = 0.0;
+    for (int yt = ya; yt < yb; yt += RB)
+        for (int y = yt + share; y < min(yt + RB, yb); y += rs)
+            for (int c = 0; c < G; c += 32) {
+                float part = 0.f;
+                for (int x = c; x < min(c + 32, G); ++x)
+                    part = fmaf(sample(a, (size_t)(y0 + y) * W + x0 + x), rw[y * G + x], part);
+                t += (double)part;
+            }
+    return t;
+}
+
 template <typename In>
 __global__ void __launch_bounds__(TRACK_THREADS, 2)
 k_track_cc(const In* __restrict__ frames, int W, int H, int x0, int y0, int G, int S, TrackShape sh,
@@ -297,10 +317,20 @@ k_track_cc(const In* __restrict__ frames, int W, int H, int x0, int y0, int G, i
     double* const red = reinterpret_cast<double*>(smem);                 // [rs][n][ng * SG]
     double* const mine = red + (size_t)sh.rs * sh.slots * SG;            // [n][n]
     const int cw = sh.ng * SG;
-    if (work)
+    if (work) {
+        double* const own = red + ((size_t)share * n + syi) * cw + s0;
+        bool finite = true;
 #pragma unroll
-        for (int k = 0; k < SG; ++k)                                     // an infinite sum leaves no low part
-            red[((size_t)share * n + syi) * cw + s0 + k] = isfinite(hi[k]) ? (double)hi[k] + (double)lo[k] : (double)hi[k];
+        for (int k = 0; k < SG; ++k) {
+            own[k] = (double)hi[k] + (double)lo[k];
+            finite = finite && (s0 + k >= n || isfinite(hi[k]));
+        }
+        // a chunk that is not finite, or a sum past the range of a float: this
+        // thread's chunks once more, summed in FP64
+        if (std::is_same<In, float>::value && !finite)
+            for (int k = 0; k < SG && s0 + k < n; ++k)
+                own[k] = row_share_fp64(a, W, x0 + s0 + k - S, y0 + syi - S, G, ya, yb, share, sh.rs, rw);
+    }
     __syncthreads();
     for (int k = tid; k < n * n; k += nt) {
         const int j = k / n, i = k - j * n;
