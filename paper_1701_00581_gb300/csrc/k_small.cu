@@ -139,7 +139,8 @@ k_stats(PlanDev p, const void* __restrict__ spec, int F, float* __restrict__ P,
 // subfields: the factor T0 / sqrt(max(STF, 1e-4)) is formed once in FP64 and
 // split in two floats, and per subfield the difference, the root and the
 // product run on pairs of floats (GB300's FP64 unit would take 0.2 ms for the
-// 3.3 M values of a TiO burst; this takes 35 us).
+// 3.3 M values of a TiO burst; this takes 35 us).  Values whose pairs would run
+// out of a float's range take the formula in FP64.
 __global__ void __launch_bounds__(256)
 k_amplitude(PlanDev p, int nsub, const double* __restrict__ stf, const float* __restrict__ P,
             const float* __restrict__ noise, float* __restrict__ A) {
@@ -152,8 +153,10 @@ k_amplitude(PlanDev p, int nsub, const double* __restrict__ stf, const float* __
     const double t0 = p.t0[o];
     const bool dc = kx == 0 && ky == 0, in = t0 > 0.0;
     float gh = 0.f, gl = 0.f;
+    double s = 1.0;
     if (in) {
-        const double g = t0 / sqrt(fmax(stf[(size_t)(ky + p.N / 2) * p.N + kx + p.N / 2], 1e-4));
+        s = fmax(stf[(size_t)(ky + p.N / 2) * p.N + kx + p.N / 2], 1e-4);
+        const double g = t0 / sqrt(s);
         gh = (float)g;
         gl = (float)(g - (double)gh);
     }
@@ -166,15 +169,16 @@ k_amplitude(PlanDev p, int nsub, const double* __restrict__ stf, const float* __
             const float x = P[(size_t)sl * hb + o], y = -noise[sl];
             const float hi = __fadd_rn(x, y), bb = __fsub_rn(hi, x);
             const float lo = __fadd_rn(__fsub_rn(x, __fsub_rn(hi, bb)), __fsub_rn(y, bb));
-            if (hi == INFINITY) {
-                a = INFINITY;
-            } else if (hi > 0.f) {                   // a NaN counts as no power, as the maximum has it
-                const float r = sqrtf(hi);
-                // the rest of the root (0 where the difference is too small
-                // for its residual to be represented), then (r + c)(gh + gl)
-                const float c = hi > 1e-30f ? __fdiv_rn(__fadd_rn(__fmaf_rn(-r, r, hi), lo), 2.f * r) : 0.f;
-                const float q = __fmul_rn(r, gh);
-                a = __fadd_rn(q, __fmaf_rn(c, gh, __fmaf_rn(r, gl, __fmaf_rn(r, gh, -q))));
+            if (hi > 0.f) {                          // a NaN counts as no power, as the maximum has it
+                const float r = sqrtf(hi), q = __fmul_rn(r, gh);
+                if (hi >= 1e-30f && hi < INFINITY && fminf(q, gh) >= 1e-30f) {
+                    // the rest c of the root, then (r + c)(gh + gl): every term
+                    // dropped or rounded is below 2^-44 q, and a float holds it
+                    const float c = __fdiv_rn(__fadd_rn(__fmaf_rn(-r, r, hi), lo), 2.f * r);
+                    a = __fadd_rn(q, __fmaf_rn(c, gh, __fmaf_rn(r, gl, __fmaf_rn(r, gh, -q))));
+                } else {
+                    a = (float)(sqrt(fmax((double)x + (double)y, 0.0) / s) * t0);
+                }
             }
         }
         A[(size_t)sl * hb + o] = a;
