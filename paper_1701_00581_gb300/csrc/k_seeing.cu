@@ -113,7 +113,9 @@ k_seeing(PlanDev p, int F, int sub0, const float* __restrict__ P, const float2* 
     for (int w = 1; w < SE_THREADS / 32; ++w) n = min(n, fail[w]);
     // FP32 cost of candidate tid and a bound on its error: the exponent's
     // rounding (|6.88 (rho x)^(5/3)| < 104 where e > 0, three roundings) moves
-    // the model by less than 2.2e-5 of its value <= 1, taken as 4e-5
+    // the model by less than 2.2e-5 of its value <= 1, taken as 4e-5.  Where e
+    // is denormal the model is below 2e-8 itself, unless a is as small: such a
+    // candidate (a constant ck that hardly differs from 0) goes to FP64 unscreened
     const double2 c = p.cand[tid];
     float j32 = 0.f, ad = 0.f;
     {
@@ -126,6 +128,7 @@ k_seeing(PlanDev p, int F, int sub0, const float* __restrict__ P, const float2* 
             ad += fabsf(d);
         }
     }
+    if (c.y > 0.0 && c.y < 1e-30) j32 = NAN;
     const float err = 8e-5f * ad + 2e-9f * n + 1e-5f * j32;
     float up = j32 + err;                          // a NaN drops out of the minimum
     if (!(up == up)) up = INFINITY;
