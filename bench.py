@@ -408,7 +408,7 @@ def run_batched(torch, plan, frames, spec, F, n_sub, info, args, stream, peak):
     del fgraph
     fused = {"launch_ms_per_burst": round(f0.elapsed_time(f1) / (args.steps * nb), 3),
              "bursts_per_s": round(nb * args.steps / (f1.elapsed_time(f2) / 1000.0), 4),
-             "items": bf.info["n_items"], "ctas": bf.info["grid"], "opts": dict(bf.opts),
+             "transforms_and_tiles": bf.info["n_items"], "ctas": bf.info["grid"], "opts": dict(bf.opts),
              "status_ok": bf.status() == 0,
              "note": "SM_BATCH_FUSED: every transform and tile of the batch from one device queue; the whole "
                      "batch captured in a CUDA graph and replayed per step"}

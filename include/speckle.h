@@ -363,9 +363,9 @@ typedef struct {
                            SM_BATCH_GRID: the transforms first, then one grid
                            of CTAs over every tile of every burst (scheduled
                            by the hardware, not a queue)                      */
-    int tile_order;     /* order of a subfield's tiles in the queue: 1 as the
-                           plan lists them (by target block), 2 costliest
-                           first                                               */
+    int tile_order;     /* order of a subfield's bispectrum tasks in the queue:
+                           1 by strip of targets and block of offsets, 2 as
+                           the plan lists them, costliest first                */
 } sm_batch_opts;
 
 /* Build the work queue of a batch of n (1..8) bursts: burst i has the plan
@@ -373,9 +373,11 @@ typedef struct {
  * frame size, N, R) but share the device and the spectra precision, and
  * accumulate plain FP32 sums (SM_ACC_PLAIN).  The queue holds one item per
  * (burst, subfield, frame) transform (SM_BATCH_FUSED) and per (burst,
- * subfield, tile) of the bispectrum (SM_BATCH_FUSED, SM_BATCH_TILES); a
- * subfield's transforms come `lookahead` subfields ahead of its tiles.  The
- * SM_BATCH_GRID launch needs no queue.  opts may be NULL
+ * subfield, task) of the bispectrum (SM_BATCH_FUSED, SM_BATCH_TILES; a task
+ * computes the used pairs of up to 128 rows of four targets and one block of
+ * offsets, from one tile or several); a subfield's transforms come
+ * `lookahead` subfields ahead of its tasks.  The SM_BATCH_GRID launch needs
+ * no queue.  opts may be NULL
  * (all tuned).  Allocates the queue, the dependency counters and a
  * transform scratch tile per persistent CTA on the device (sm_batch_info
  * reports the bytes), and one stream per burst for the stages after the
@@ -388,8 +390,9 @@ int sm_batch_create(int n, const sm_plan* const* plans, const int* F, const int*
 /* The shape the batch was built with (the tuned values filled in).         */
 int sm_batch_get_opts(const sm_batch* bt, sm_batch_opts* opts);
 int sm_batch_destroy(sm_batch* bt);
-/* Transforms and tiles that the queue covers (SM_BATCH_GRID: 0), persistent
- * CTAs of the launch, device bytes held.                                    */
+/* Transforms and tiles that the queue's items cover (SM_BATCH_GRID: 0; not
+ * the number of items: a task holds pairs of several tiles, a tile's pairs
+ * may go to several tasks), persistent CTAs of the launch, device bytes held. */
 int sm_batch_info(const sm_batch* bt, int* n_items, int* grid, size_t* device_bytes);
 
 /* The batched transforms and bispectrum alone: spectra, flux and mean of

@@ -153,7 +153,7 @@ def main():
         for r in sorted(rows, key=lambda r: r["ms_per_burst"]):
             mark = " **(chosen)**" if r is win else ""
             out.append(f"| {r['lookahead']} | {r['ctas_per_sm']} | {LAUNCH_NAMES[r['launch']]} "
-                       f"| {'plan' if r['tile_order'] == 1 else 'costliest first'} | {r['ms_per_burst']:.4g}{mark} |")
+                       f"| {'by strip' if r['tile_order'] == 1 else 'costliest first'} | {r['ms_per_burst']:.4g}{mark} |")
         out.append("")
     text = "\n".join(out)
     print(text)

@@ -21,7 +21,7 @@ struct sm_batch {
     std::vector<const sm_plan*> plans;
     std::vector<int> F, frame_type, cnt_base;
     int n_cnt = 0, n_items = 0, grid = 0;
-    int n_work = 0;                     // transforms and tiles that the queue covers
+    int n_work = 0;                     // transforms and tiles that the queue's items cover
     size_t smem = 0, scr_elems = 0;
     int4* d_items = nullptr;
     int* d_state = nullptr;             // [0] queue head, [1] status, [2..] per-subfield counters
