@@ -121,6 +121,28 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def distinct_products(K: int, r2: float, R: int) -> int:
+    """Triple products a subfield's bispectrum needs: the used pairs (w, v), less one of the two orders of a pair
+    whose offsets v and w - v both lie within R (B(u, v) = B(v, u))."""
+    r2 = int(np.floor(r2))
+    wy, wx = np.mgrid[0:K + 1, -K:K + 1]
+    w2 = wx * wx + wy * wy
+    ok = ((wy > 0) | (wx > 0)) & (w2 >= 2) & (w2 <= r2)
+    wx, wy, w2 = wx[ok], wy[ok], w2[ok]
+    n = 0
+    for vy in range(-R, R + 1):
+        for vx in range(-R, R + 1):
+            v2 = vx * vx + vy * vy
+            if not 0 < v2 <= R * R:
+                continue
+            ux, uy = wx - vx, wy - vy
+            u2 = ux * ux + uy * uy
+            used = (v2 < w2) & (u2 < w2)
+            other = (u2 <= R * R) & ((uy < vy) | ((uy == vy) & (ux < vx)))     # counted at the other order
+            n += int((used & ~other).sum())
+    return n
+
+
 # ---------------------------------------------------------------------------- CPU oracle
 def _oracle_subfield_task(task):
     """One host core's share of the CPU baseline: the FP64 oracle on one
@@ -413,7 +435,7 @@ def run_batched(torch, plan, frames, spec, F, n_sub, info, args, stream, peak):
              "note": "SM_BATCH_FUSED: every transform and tile of the batch from one device queue; the whole "
                      "batch captured in a CUDA graph and replayed per step"}
     bf.close()
-    triples = info["n_pairs"] * F * n_sub * nb
+    triples = distinct_products(info["K"], (plan.ch.fc * info["N"]) ** 2, info["R"]) * F * n_sub * nb
     ach = FLOPS_PER_TRIPLE * triples / (kms / 1000.0) / 1e12
     rec = {"value": round(nb * args.steps / (ms / 1000.0), 4), "unit": "bursts/s", "bursts_per_launch": nb,
            "ms_per_burst": round(ms / (nb * args.steps), 3), "status_ok": ok,
@@ -421,7 +443,8 @@ def run_batched(torch, plan, frames, spec, F, n_sub, info, args, stream, peak):
            "persistent_fused": fused,
            "launch_roofline": {"bound": "alu", "achieved": round(ach, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
                                "frac": round(ach / peak, 4),
-                               "note": "bispectrum flops only (14 x used triples); the launch also does every FFT"},
+                               "note": "bispectrum flops only (14 x distinct triple products); the launch also does every "
+                                       "FFT"},
            "note": f"{nb} copies of the burst in separate workspaces per batched spectra + bispectrum launch "
                    "(the autotuned shape), then each burst's remaining stages, the whole batch captured once in a "
                    "CUDA graph and replayed per step; inputs resident in HBM"}
@@ -636,7 +659,7 @@ def main():
     value = whole_job_rate(args.steps, world, ms_max / 1000.0)
 
     # roofline of the dominant kernel (bispectrum): FP32 ALU bound
-    triples = info["n_pairs"] * F * n_sub
+    triples = distinct_products(info["K"], (plan.ch.fc * info["N"]) ** 2, info["R"]) * F * n_sub
     achieved = FLOPS_PER_TRIPLE * triples / (bisp_ms / 1000.0) / 1e12
     props = torch.cuda.get_device_properties(local)
     peaks_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -649,7 +672,9 @@ def main():
                 "frac": round(achieved / peak, 4),
                 "traffic": None if traffic is None else int(traffic),
                 "kernel": "k_bispectrum", "kernel_ms": round(bisp_ms, 3),
-                "note": (f"{FLOPS_PER_TRIPLE} flops x {triples:.3e} used triples per launch; peak = "
+                "note": (f"{FLOPS_PER_TRIPLE} flops x {triples:.3e} distinct triple products per launch "
+                         f"({info['n_pairs'] * F * n_sub:.3e} used: a pair with both offsets within R is multiplied "
+                         f"once and stored twice); peak = "
                          f"{props.multi_processor_count} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x "
                          f"{sm_max:.0f} MHz")}
 
