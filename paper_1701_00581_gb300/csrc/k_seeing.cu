@@ -111,6 +111,10 @@ k_seeing(PlanDev p, int F, int sub0, const float* __restrict__ P, const float2* 
     int n = fail[0];
 #pragma unroll
     for (int w = 1; w < SE_THREADS / 32; ++w) n = min(n, fail[w]);
+    if (n == 0) {                                  // no usable annulus: nothing to fit (n is the same in every thread)
+        if (tid == 0) seeing[cube] = SE_HI;
+        return;
+    }
     // FP32 cost of candidate tid and a bound on its error: the exponent's
     // rounding (|6.88 (rho x)^(5/3)| < 104 where e > 0, three roundings) moves
     // the model by less than 2.2e-5 of its value <= 1, taken as 4e-5.  Where e
@@ -181,20 +185,16 @@ k_seeing(PlanDev p, int F, int sub0, const float* __restrict__ P, const float2* 
     if (tid == 0) {
         for (int w = 1; w < SE_THREADS / 32; ++w)
             if (num[w] < best || (num[w] == best && bi[w] < im)) best = num[w], im = bi[w];
-        double xhat = SE_HI;
-        if (n > 0) {
-            const double llo = log(SE_LO), lhi = log(SE_HI);
-            double t = log_candidate(llo, lhi, im);
-            if (im > 0 && im < SE_GRID - 1) {
-                const double curv = J[im - 1] - 2.0 * J[im] + J[im + 1];
-                if (curv > 0.0) {
-                    const double h = log_candidate(llo, lhi, 1) - log_candidate(llo, lhi, 0);
-                    t += 0.5 * h * (J[im - 1] - J[im + 1]) / curv;
-                }
+        const double llo = log(SE_LO), lhi = log(SE_HI);
+        double t = log_candidate(llo, lhi, im);
+        if (im > 0 && im < SE_GRID - 1) {
+            const double curv = J[im - 1] - 2.0 * J[im] + J[im + 1];
+            if (curv > 0.0) {
+                const double h = log_candidate(llo, lhi, 1) - log_candidate(llo, lhi, 0);
+                t += 0.5 * h * (J[im - 1] - J[im + 1]) / curv;
             }
-            xhat = exp(t);
         }
-        seeing[cube] = xhat;
+        seeing[cube] = exp(t);
     }
 }
 
