@@ -9,7 +9,7 @@ namespace {
 using smi::PlanDev;
 
 constexpr int STAT_THREADS = 256;
-constexpr int STAT_CTAS = 8;           // CTAs (one cluster) per subfield
+constexpr int STAT_CTAS = 8;           // CTAs (one cluster) per subfield at most
 constexpr int STAT_LOADS = 10;         // frames whose loads are in flight together
 
 // Two neighbouring spectrum values as stored, and as floats.
@@ -33,7 +33,7 @@ template <int PREC> __device__ __forceinline__ float4 pair_values(uint2 v) {
 
 // P = <|I_i|^2>, M = <I_i> over the F frames on the half box ky = 0..K;
 // noise = mean of P over {ky >= 1, |k|^2 > r^2} (the half-box corners).
-// HBM bound: a cluster of 8 CTAs per subfield streams its F spectra once,
+// HBM bound: a cluster of up to 8 CTAs per subfield streams its F spectra once,
 // each thread summing two neighbouring values over the frames in order
 // (16-byte loads of FP32 spectra, ten frames in flight: a single subfield is
 // bound by the latency of its chain of loads).  The corners' sum runs over a
@@ -43,12 +43,12 @@ template <int PREC> __device__ __forceinline__ float4 pair_values(uint2 v) {
 // flight.
 template <int PREC>
 __global__ void __launch_bounds__(STAT_THREADS)
-k_stats(PlanDev p, const void* __restrict__ spec, int F, float* __restrict__ P,
+k_stats(PlanDev p, int ctas, const void* __restrict__ spec, int F, float* __restrict__ P,
         float2* __restrict__ M, float* __restrict__ noise) {
     using PT = typename Pair<PREC>::T;
     __shared__ double red_s[STAT_THREADS / 32], part_s;
     __shared__ int red_n[STAT_THREADS / 32], part_n;
-    const int sl = blockIdx.x / STAT_CTAS, part = blockIdx.x % STAT_CTAS, tid = threadIdx.x;
+    const int sl = blockIdx.x / ctas, part = blockIdx.x - sl * ctas, tid = threadIdx.x;
     const size_t box2 = (size_t)p.box_rows * p.box_pitch / 2;
     const size_t hb = (size_t)p.hb_rows * p.box_pitch;
     // the pitch is a multiple of 4; the last value of a row pairs with the
@@ -58,7 +58,7 @@ k_stats(PlanDev p, const void* __restrict__ spec, int F, float* __restrict__ P,
     const float invF = 1.0f / (float)F;
     double cs = 0.0;
     int cn = 0;
-    for (int e = part * STAT_THREADS + tid; e < ne2; e += STAT_CTAS * STAT_THREADS) {
+    for (int e = part * STAT_THREADS + tid; e < ne2; e += ctas * STAT_THREADS) {
         const int ky = e / hp, col = 2 * (e - ky * hp);
         float ps0 = 0.f, ps1 = 0.f;
         float2 m0 = make_float2(0.f, 0.f), m1 = make_float2(0.f, 0.f);
@@ -117,7 +117,7 @@ k_stats(PlanDev p, const void* __restrict__ spec, int F, float* __restrict__ P,
     if (part == 0 && tid == 0) {
         double s = 0.0;
         int n = 0;
-        for (unsigned c = 0; c < STAT_CTAS; ++c) {
+        for (int c = 0; c < ctas; ++c) {
             unsigned as = (unsigned)__cvta_generic_to_shared(&part_s), an = (unsigned)__cvta_generic_to_shared(&part_n);
             double ps;
             int pn;
@@ -309,16 +309,19 @@ template <int PREC>
 cudaError_t stats_go(const smi::PlanDev& p, const void* spec, int F, int nsub, float* P, float2* M, float* noise,
                      cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nsub * STAT_CTAS);
+    // as many CTAs as hold a value each per thread; more would only wait for the
+    // others at the cluster's barriers (225 subfields of 64^2: 70 us with 8)
+    const int ctas = std::min(STAT_CTAS, (p.hb_rows * p.box_pitch / 2 + STAT_THREADS - 1) / STAT_THREADS);
+    cfg.gridDim = dim3(nsub * ctas);
     cfg.blockDim = dim3(STAT_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = STAT_CTAS;
+    at.val.clusterDim.x = ctas;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_stats<PREC>, p, spec, F, P, M, noise);
+    return cudaLaunchKernelEx(&cfg, k_stats<PREC>, p, ctas, spec, F, P, M, noise);
 }
 
 int sm_count() {
