@@ -1,0 +1,48 @@
+"""The bispectrum's fixed costs: what a launch takes beside the products of its frames."""
+from __future__ import annotations
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _ms(F, stage="bispectrum", reps=40, graph=False, **kw):
+    """Time of `reps` launches, the best of five groups; with `graph` replayed from a CUDA graph, without the host."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("no CUDA device")
+    from paper_1701_00581_gb300 import Channel, Plan
+    plan = Plan(Channel(max_frames=F, **kw))
+    n = plan.info["n_sub"]
+    ws, lay = plan.workspace(F, n)
+    ws.zero_()
+    s = torch.cuda.Stream()
+    one = getattr(plan, "stage_" + stage)
+
+    def run():
+        for _ in range(reps):
+            one(F, n, ws, lay, s)
+    with torch.cuda.stream(s):
+        run()
+        torch.cuda.synchronize()
+        if graph:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                run()
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            a.record(s)
+            g.replay() if graph else run()
+            b.record(s)
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+    return min(t[1:])
+
+
+def test_one_frame_is_a_few_latencies():
+    """One frame of one 64^2 subfield is a chain of memory latencies, as the statistics of one frame are: less than
+    twice their time (2.3 times with a latency more for every pair stored in both orders)."""
+    kw = dict(W=64, H=64, N=64, R=8, graph=True)
+    assert _ms(1, **kw) < 2.0 * _ms(1, "stats", **kw)
