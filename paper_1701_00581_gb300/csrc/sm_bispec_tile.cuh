@@ -135,7 +135,7 @@ __device__ __forceinline__ float2 raw_to_float2(unsigned w) {
     if (PREC == SM_FP16) {
         return __half22float2(*reinterpret_cast<const __half2*>(&w));      // still scaled
     } else {
-        return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w));
+        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
     }
 }
 

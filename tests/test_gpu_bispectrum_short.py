@@ -46,3 +46,10 @@ def test_one_frame_is_a_few_latencies():
     twice their time (2.3 times with a latency more for every pair stored in both orders)."""
     kw = dict(W=64, H=64, N=64, R=8, graph=True)
     assert _ms(1, **kw) < 2.0 * _ms(1, "stats", **kw)
+
+
+def test_bfloat16_costs_what_half_does():
+    """The two storage types differ in their conversion alone, a shift against an instruction."""
+    from paper_1701_00581_gb300 import SM_ACC_KAHAN, SM_BF16, SM_FP16
+    kw = dict(W=512, H=512, N=256, R=24, acc_mode=SM_ACC_KAHAN, reps=2)
+    assert _ms(30, spectra_prec=SM_BF16, **kw) < 1.02 * _ms(30, spectra_prec=SM_FP16, **kw)
