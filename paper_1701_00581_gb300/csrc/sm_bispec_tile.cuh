@@ -228,26 +228,22 @@ __device__ __forceinline__ void bispec_tile(const PlanDev& p, const void* __rest
         nb[i] = nb[i] * E / 8;
         g[i] = sp + src;
     }
-    auto copy = [&](unsigned soff, size_t goff, bool in) {
+    auto copy = [&](unsigned soff, size_t goff) {
 #pragma unroll
         for (int i = 0; i < SLOTS; ++i)
-            if (dst[i] >= 0) cp_pair<E>(s0 + dst[i] * E + soff, g[i] + goff, in ? nb[i] : 0);
+            if (dst[i] >= 0) cp_pair<E>(s0 + dst[i] * E + soff, g[i] + goff, nb[i]);
     };
-    // Stage st holds frames FB st .. FB st + FB - 1; frames past F are
-    // zero-filled (no global read) so that every stage is multiplied out whole.
+    // Stage st holds frames FB st .. FB st + FB - 1, the last one those up to F.
     auto issue = [&](int st) {
         if (st < nst) {
             const unsigned sb = (unsigned)((st & 1) * FB * BUF * E);
             if (st * FB + FB <= F) {
 #pragma unroll
                 for (int ff = 0; ff < FB; ++ff)
-                    copy(sb + ff * BUF * E, (size_t)(st * FB + ff) * box, true);
+                    copy(sb + ff * BUF * E, (size_t)(st * FB + ff) * box);
             } else {
-#pragma unroll
-                for (int ff = 0; ff < FB; ++ff) {
-                    const bool in = st * FB + ff < F;
-                    copy(sb + ff * BUF * E, in ? (size_t)(st * FB + ff) * box : 0, in);
-                }
+#pragma unroll 1
+                for (int ff = 0; ff < F - st * FB; ++ff) copy(sb + ff * BUF * E, (size_t)(st * FB + ff) * box);
             }
         }
         asm volatile("cp.async.commit_group;");
@@ -312,8 +308,9 @@ __device__ __forceinline__ void bispec_tile(const PlanDev& p, const void* __rest
         const int ou = OFF_U + (wyl - warp + smi::VBY - 1) * PU + 4 * gx + smi::VBX - col0 - NC;
         for (int st = 0; st < nst; ++st) {
             const float2* Sst = next_stage(st);
+            const int nf = min(FB, F - st * FB);
 #pragma unroll 1
-            for (int ff = 0; ff < FB; ++ff) {
+            for (int ff = 0; ff < nf; ++ff) {
                 const float2* const Sf = Sst + ff * BUF;
                 if constexpr (KAHAN) accumulate_frame<NC, VCH>(Sf + ow, Sf + ou, Sf + ov, part);
                 else accumulate_frame<NC, VCH>(Sf + ow, Sf + ou, Sf + ov, acc);

@@ -53,3 +53,12 @@ def test_bfloat16_costs_what_half_does():
     from paper_1701_00581_gb300 import SM_ACC_KAHAN, SM_BF16, SM_FP16
     kw = dict(W=512, H=512, N=256, R=24, acc_mode=SM_ACC_KAHAN, reps=2)
     assert _ms(30, spectra_prec=SM_BF16, **kw) < 1.02 * _ms(30, spectra_prec=SM_FP16, **kw)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_last_stage_holds_its_frames_alone(prec):
+    """Nine frames take as many stages as twelve (FP16: seven as nine), three; what the last one lacks is neither
+    staged nor multiplied, so they take 9/12 (7/9) of the products' time."""
+    kw = dict(W=512, H=512, N=128, R=16, spectra_prec=prec)
+    few, all_ = (7, 9) if prec else (9, 12)
+    assert _ms(few, **kw) < 0.93 * _ms(all_, **kw)
