@@ -381,6 +381,16 @@ __device__ __forceinline__ void bispec_tile(const PlanDev& p, const void* __rest
     };
 #pragma unroll
     for (int pass = 0; pass < NP; ++pass) {
+        if constexpr (KAHAN) {                     // a pass that no warp has a column in (the same for all warps)
+            const unsigned ranges = __reduce_or_sync(0xffffffffu, (unsigned)T2.y);
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < smi::VBY; ++q) {
+                const int f = ranges >> (8 * q) & 15, c = ranges >> (8 * q + 4) & 15;
+                any |= c > 0 && f < (pass + 1) * NCP && f + c > pass * NCP;
+            }
+            if (!any) continue;
+        }
         __syncwarp();                              // a warp's idle lanes leave run() before the others
         if (pass > 0) __syncthreads();             // the previous pass is done with the ring
         issue(0);

@@ -62,3 +62,11 @@ def test_last_stage_holds_its_frames_alone(prec):
     kw = dict(W=512, H=512, N=128, R=16, spectra_prec=prec)
     few, all_ = (7, 9) if prec else (9, 12)
     assert _ms(few, **kw) < 0.93 * _ms(all_, **kw)
+
+
+def test_compensated_sums_skip_an_empty_pass():
+    """R = 1: every offset lies in a block's first four columns, so the compensated sums stream the frames once, as
+    the plain ones do (twice: about twice the time)."""
+    from paper_1701_00581_gb300 import SM_ACC_KAHAN
+    kw = dict(W=512, H=512, N=128, R=1)
+    assert _ms(100, acc_mode=SM_ACC_KAHAN, **kw) < 1.6 * _ms(100, **kw)
