@@ -51,6 +51,7 @@ using smi::TILE_PAIRS;
 
 constexpr int PH_WARPS = 16, TH = 32 * PH_WARPS;   // warps and threads of a CTA
 constexpr int PH_STEPS = 8;            // steps of 4 tile rows whose B loads are in flight together
+constexpr int PH_SNR_STEPS = 4;        // the same with SNR weights, whose P loads are in flight as well
 constexpr int PH_LATE_WARPS = 8;       // warps that walk the rings (a ring has 4 to 6 points on average)
 
 // Complex values of the recursion's arithmetic type T.
@@ -253,13 +254,11 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
     }
 
     const float* const Ps = P + (size_t)sl * hb;   // power spectrum, for the SNR weighting
-    auto pget = [&](int i) -> T {                  // P at signed index i; P(-k) = P(k)
-        const int a = abs(i) / ZB, ky = (a + zp / 2) / zp, kx = a - ky * zp;
-        return (T)__ldg(Ps + ky * p.box_pitch + kx + K);
-    };
+    auto pget = [&](int i) { return __ldg(Ps + abs(i) / ZB + K); };    // P at signed index i (box pitch); P(-k) = P(k)
     const float2* const Bs = B + (size_t)sl * p.n_tiles * TILE_PAIRS;
-    // s += z(u) z(v) conj b, weighted, for the split of w (index iw) by v (iv)
-    auto add_term = [&](T& sx, T& sy, float2 b, int iw, int iv) {
+    // s += z(u) z(v) conj b, weighted, for the split of w (index iw) by v (iv);
+    // SNR weights: p2 = P(u), P(v)
+    auto add_term = [&](T& sx, T& sy, float2 b, int iw, int iv, float2 p2) {
         const T bx = (T)b.x, by = (T)b.y;
         const T2 zu = zget(zs, iw - iv);
         const T2 zv = zget(zs, iv);
@@ -276,7 +275,7 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
             // the divisor of the term: |B|, or the speckle-noise variance of B
             T den;
             if constexpr (WEIGHT == SM_W_UNIT) den = sqrt(bx * bx + by * by);
-            else den = pget(iw - iv) * pget(iv) * pget(iw);
+            else den = (T)p2.x * (T)p2.y * (T)pget(iw);
             if (den > (T)0) {
                 sx += (c.x * bx + c.y * by) / den;
                 sy += (c.y * bx - c.x * by) / den;
@@ -311,7 +310,7 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
             T sx = 0, sy = 0;
             auto rows = [&](auto steps, int g) {           // 4 rows a step
                 constexpr int ST = decltype(steps)::value;
-                float2 b[ST];
+                float2 b[ST], p2[ST];
                 int iv[ST];
 #pragma unroll
                 for (int i = 0; i < ST; ++i) {
@@ -320,12 +319,19 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
                     b[i] = make_float2(0.f, 0.f);
                     if (ok) b[i] = __ldcs(Bw + (size_t)e.x * smi::VBX);
                     iv[i] = ok ? (e.y >> 8) + l8 * ZB : 0;        // otherwise adds z(w) conj 0
+                    p2[i] = make_float2(0.f, 0.f);
+                    if (WEIGHT == SM_W_SNR && ok) p2[i] = make_float2(pget(rec.x - iv[i]), pget(iv[i]));
                 }
 #pragma unroll
-                for (int i = 0; i < ST; ++i) add_term(sx, sy, b[i], rec.x, iv[i]);
+                for (int i = 0; i < ST; ++i) add_term(sx, sy, b[i], rec.x, iv[i], p2[i]);
             };
-            if (n > 16) rows(std::integral_constant<int, PH_STEPS>{}, 0);
-            else rows(std::integral_constant<int, PH_STEPS / 2>{}, 0);
+            if constexpr (WEIGHT == SM_W_SNR) {
+#pragma unroll 1
+                for (int g = 0; g < n; g += 4 * PH_SNR_STEPS) rows(std::integral_constant<int, PH_SNR_STEPS>{}, g);
+            } else {
+                if (n > 16) rows(std::integral_constant<int, PH_STEPS>{}, 0);
+                else rows(std::integral_constant<int, PH_STEPS / 2>{}, 0);
+            }
             reduce_warp(sx, sy);
             const T2 s = Cx<T>::make(sx, sy);
             if (cl == 1) {
@@ -438,8 +444,13 @@ k_phase(PlanDev p, const float2* __restrict__ B, const float2* __restrict__ M, c
             };
             auto finish = [&](const Point& t) {
                 T sx = t.s.x, sy = t.s.y;
-                if (t.a < t.end) add_term(sx, sy, t.b, t.iw, t.iv);
-                for (int a = t.a + 32; a < t.end; a += 32) add_term(sx, sy, lb[a], t.iw, liv[a]);
+                auto late_term = [&](float2 b, int iv) {
+                    float2 p2 = make_float2(0.f, 0.f);
+                    if (WEIGHT == SM_W_SNR) p2 = make_float2(pget(t.iw - iv), pget(iv));
+                    add_term(sx, sy, b, t.iw, iv, p2);
+                };
+                if (t.a < t.end) late_term(t.b, t.iv);
+                for (int a = t.a + 32; a < t.end; a += 32) late_term(lb[a], liv[a]);
                 reduce_warp(sx, sy);
                 const T n2 = sx * sx + sy * sy;
                 T2 zz = Cx<T>::make(1, 0);

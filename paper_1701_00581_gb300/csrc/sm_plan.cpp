@@ -459,10 +459,13 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     //
     // The phasor table's pitch is 8 (mod 16) complex floats, so that the two
     // rows of offsets that half a warp reads fall on different banks; wider
-    // values, or a table that would not fit, take the box's own pitch.
+    // values, or a table that would not fit, take the box's own pitch, and so
+    // does the SNR weighting, whose terms read the power spectrum at the same
+    // indices (with another pitch each would take a division: 225 subfields of
+    // 256^2 20.2 ms).
     int per_batch = std::max(PHASE_BATCH_MIN, std::min(PHASE_BATCH_MAX, d.n_points / 32));
     d.zpitch = d.box_pitch;
-    if (d.phase_prec == SM_PHASE_FP32) {
+    if (d.phase_prec == SM_PHASE_FP32 && d.weight != SM_W_SNR) {
         const int padded = (2 * K + 2 + 7) / 16 * 16 + 8;
         const int most_units = per_batch * (nvb * VBY / 32 + 1);
         if (smk::phase_smem_bytes(d.hb_rows, padded, per_batch, most_units, PHASE_LATE, d.phase_prec) <= 227 * 1024)
