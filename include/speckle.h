@@ -353,7 +353,9 @@ typedef struct {
  * batch's largest subfield size N and its R (the table the library's
  * autotuner wrote, autotune.py).                                            */
 typedef struct {
-    int lookahead;      /* subfields whose transforms run ahead of the tiles  */
+    int lookahead;      /* subfields whose transforms run ahead of the tasks
+                           (0 and SM_BATCH_FUSED: the tuned value, or twice the
+                           subfields whose items the CTAs hold at once, if more) */
     int ctas_per_sm;    /* persistent CTAs per SM: 3 (168 registers a thread)
                            or 4 (128)                                          */
     int launch;         /* SM_BATCH_FUSED: one persistent launch whose items

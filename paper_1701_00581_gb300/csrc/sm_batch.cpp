@@ -77,6 +77,7 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
     for (int i = 0; i < n; ++i)
         if (!plans[i]) { set_error("NULL plan"); return SM_EINVAL; }
     sm_batch_opts opts = opts_in ? *opts_in : sm_batch_opts{};
+    bool tuned_lookahead = false;
     {
         int N = 0, R = 0;
         for (int i = 0; i < n; ++i)
@@ -85,6 +86,7 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
                 R = plans[i]->dev.R;
             }
         const smt::TuneEntry t = smt::tune_for(N, R, opts.launch);
+        tuned_lookahead = opts.lookahead == 0;
         if (opts.lookahead == 0) opts.lookahead = t.lookahead;
         if (opts.ctas_per_sm == 0) opts.ctas_per_sm = t.ctas_per_sm;
         if (opts.launch == 0) opts.launch = t.launch;
@@ -96,7 +98,6 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
     if (opts.launch < SM_BATCH_FUSED || opts.launch > SM_BATCH_GRID) {
         set_error("launch must be SM_BATCH_FUSED, SM_BATCH_TILES or SM_BATCH_GRID"); return SM_EINVAL;
     }
-    const int lookahead = opts.lookahead;
     const bool fused = opts.launch == SM_BATCH_FUSED, queued = opts.launch != SM_BATCH_GRID;
     for (int i = 0; i < n; ++i) {
         const sm_plan* p = plans[i];
@@ -109,6 +110,18 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
         if (F[i] < 1 || F[i] > p->ch.max_frames) { set_error("F out of range 1..max_frames"); return SM_EINVAL; }
         if (frame_type[i] != SM_U16 && frame_type[i] != SM_F32) { set_error("bad frame_type"); return SM_EINVAL; }
     }
+    // The CTAs of the launch hold the items of several subfields at once when a
+    // subfield has few (64^2: 136); a task among them whose transforms are in
+    // flight as well waits for them.  So by itself the lookahead covers twice
+    // the items in flight (25 subfields of 64^2, two bursts: 4 1.12 ms, 9 0.63).
+    int nsm = 0;
+    if (fused && tuned_lookahead &&
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, plans[0]->device) == cudaSuccess)
+        for (int i = 0; i < n; ++i) {
+            const int items = F[i] + plans[i]->dev.n_bis_tasks;
+            opts.lookahead = std::max(opts.lookahead, (2 * nsm * opts.ctas_per_sm + items - 1) / items);
+        }
+    const int lookahead = opts.lookahead;
     sm_batch* bt = new (std::nothrow) sm_batch();
     if (!bt) { set_error("host allocation failed"); return SM_ENOMEM; }
     bt->n = n;
@@ -172,7 +185,6 @@ extern "C" int sm_batch_create(int n, const sm_plan* const* plans, const int* F,
         return cuda_fail(ce, where);
     };
     if (e != cudaSuccess) return fail(e, "cudaSetDevice");
-    int nsm = 0;
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, bt->device);
     if (e != cudaSuccess) return fail(e, "cudaDeviceGetAttribute");
     if (!fused) bt->smem = smk::batch_smem_bytes(0, 0, bt->prec);      // tiles only

@@ -79,7 +79,10 @@ int main(int, char** argv) {
     size_t bytes = 0;
     sm_batch_info(bt, &n_items, &grid, &bytes);
     bad += n_items != covered || bytes < (size_t)bt->n_items * sizeof(int4);
-    printf("%d wrong, %d items\n", bad, bt->n_items);
+    int least = 1 << 30;                                   // items of the smallest subfield
+    for (int b = 0; b < 3; ++b) least = std::min(least, F[b] + plans[b]->dev.n_bis_tasks);
+    printf("%d wrong, %d items, lookahead %d, in flight %d of %d a subfield\n", bad, bt->n_items, bt->opts.lookahead, grid,
+           least);
     sm_batch_destroy(bt);
     sm_plan_destroy(plans[0]);
     sm_plan_destroy(plans[1]);

@@ -1,6 +1,7 @@
 """A batch's device queue (batch_host.cpp): every transform and every bispectrum task once, transforms before the tasks
 that read them, and sm_batch_info's count of what the queue covers."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -31,3 +32,14 @@ def batch_host(tmp_path_factory):
 def test_queue(batch_host, launch, order, lookahead):
     r = subprocess.run([batch_host, str(launch), str(order), str(lookahead)], capture_output=True, text=True)
     assert r.returncode == 0 and r.stdout.startswith("0 wrong"), r.stdout
+
+
+def test_lookahead_by_default(batch_host):
+    """Left to itself a fused queue's transforms run ahead by twice the subfields whose items the CTAs hold at once, so
+    that none of those waits for another; a given lookahead stays as it is."""
+    def run(lookahead):
+        out = subprocess.run([batch_host, "1", "2", str(lookahead)], capture_output=True, text=True, check=True).stdout
+        return [int(v) for v in re.search(r"lookahead (\d+), in flight (\d+) of (\d+)", out).groups()]
+    ahead, flight, items = run(0)
+    assert flight == 4 * 152 and ahead * items >= 2 * flight > (ahead - 1) * items
+    assert run(3)[0] == 3
