@@ -35,13 +35,12 @@
 // shared memory).  W and U start at even box
 // columns (the plan places the offset grid so that they do), so they move in
 // 16-byte copies of two spectrum values, and so does V, from one value
-// earlier when its own start is odd.  A last, partial stage is padded with
-// zero-filled frames, which add nothing to the sums.  Accumulators are
-// written once per burst.
+// earlier when its own start is odd.  A last, partial stage holds its own
+// frames only.  Accumulators are written once per burst.
 //
 // 304 subfields of 256^2, R = 24, 100 frames: 102.0 -> 89.4 ms; 225 of 128^2,
-// R = 16: 11.5 -> 8.7 ms; one of 64^2, R = 8: 47 -> 42 us; 15 of 256^2 with FP16
-// spectra 6.2 -> 5.4 ms, with compensated sums too 9.0 -> 8.8 ms.
+// R = 16: 11.5 -> 8.7 ms; one of 64^2, R = 8: 47 -> 36 us; 25 of 256^2, 30 frames:
+// FP32 3.07 -> 2.70 ms, FP16 3.66 -> 3.22, with compensated sums too 5.37 -> 5.03.
 #include "sm_bispec_tile.cuh"
 
 namespace {

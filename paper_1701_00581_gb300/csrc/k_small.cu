@@ -38,9 +38,8 @@ template <int PREC> __device__ __forceinline__ float4 pair_values(uint2 v) {
 // (16-byte loads of FP32 spectra, ten frames in flight: a single subfield is
 // bound by the latency of its chain of loads).  The corners' sum runs over a
 // fixed tree of threads and CTAs.  304 subfields of 256^2, 100 frames: 0.47 ->
-// 0.40 ms; 15: 167 -> 59 us; one of
-// 64^2: 32 -> 22 us, against one CTA of 1024 threads with four frames in
-// flight.
+// 0.40 ms; 225 of 64^2 68 -> 33 us; one of 64^2 16.7 -> 12.5 us, against one CTA of
+// 1024 threads with four frames in flight.
 template <int PREC>
 __global__ void __launch_bounds__(STAT_THREADS)
 k_stats(PlanDev p, int ctas, const void* __restrict__ spec, int F, float* __restrict__ P,

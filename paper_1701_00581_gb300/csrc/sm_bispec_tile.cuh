@@ -11,7 +11,6 @@ namespace smb {
 using smi::PlanDev;
 using smi::TILE_PAIRS;
 using smi::TILE_V;
-using smi::TILE_W;
 
 // A task is up to 32 quads (4 neighbouring targets of a 16-wide strip) per
 // offset row, packed from at most BIS_ROWS rows of targets.

@@ -87,10 +87,6 @@ struct PlanDev {
     int n_bis_tasks;
     const int* ring_start;   // [n_rings + 1]
     const int2* points;      // [n_points] (wx, wy), ring-ordered
-    const int* wb_start;     // [n_wbx * n_wby + 1] CSR: tiles of each w-block
-    const int* wb_tiles;
-    // phase recursion work items: (point, tile) pairs holding at least one
-    // pair the point reads, grouped by point, points in ring order
     // phase recursion (k_phase.cu): batches of rings; per point the tile rows
     // holding its early terms and the list of its late ones; a frequency's
     // signed index is (ky * zpitch + kx) * bytes of a phasor

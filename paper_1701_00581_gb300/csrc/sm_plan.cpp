@@ -320,7 +320,6 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     pl->n_vby = (2 * R + 1 + VBY - 1) / VBY;
     const int nwb = d.n_wbx * d.n_wby, nvb = pl->n_vbx * pl->n_vby;
     pl->tile_of.assign((size_t)nwb * nvb, -1);
-    std::vector<int> wb_count(nwb, 0);
     std::vector<QuadMask> quads((size_t)nwb * nvb * WBY * (WBX / 4));
     d.n_vbx = pl->n_vbx;
     d.n_vby = pl->n_vby;
@@ -358,7 +357,6 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
             pl->tiles.push_back(make_int4(-K + WBX * (wb % d.n_wbx), WBY * (wb / d.n_wbx),
                                           d.v_org + VBX * (vb % pl->n_vbx), -R + VBY * (vb / pl->n_vbx)));
             pl->tile_masks.push_back(masks[t]);
-            wb_count[wb]++;
         }
     d.n_tiles = (int)pl->tiles.size();
 
@@ -416,17 +414,6 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
             set_error("internal: bispectrum tile not on an even box column"); return SM_EINVAL;
         }
     pl->n_pairs = npairs;
-    pl->wb_start.assign(nwb + 1, 0);
-    for (int b = 0; b < nwb; ++b) pl->wb_start[b + 1] = pl->wb_start[b] + wb_count[b];
-    pl->wb_tiles.resize(d.n_tiles);
-    {
-        std::vector<int> fill(pl->wb_start.begin(), pl->wb_start.end() - 1);
-        for (int t = 0; t < d.n_tiles; ++t) {
-            const int4 T = pl->tiles[t];
-            const int wb = (T.y / WBY) * d.n_wbx + (T.x + K) / WBX;
-            pl->wb_tiles[fill[wb]++] = t;
-        }
-    }
 
     // recursion schedule: points of the half-plane disk with |w|^2 >= 2,
     // rings of equal |w|^2 in ascending order
@@ -645,8 +632,8 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {pl->tiles.data(), pl->tiles.size() * sizeof(int4), 0},
         {pl->ring_start.data(), pl->ring_start.size() * sizeof(int), 0},
         {pl->points.data(), pl->points.size() * sizeof(int2), 0},
-        {pl->wb_start.data(), pl->wb_start.size() * sizeof(int), 0},
-        {pl->wb_tiles.data(), pl->wb_tiles.size() * sizeof(int), 0},
+        {pl->units.data(), pl->units.size() * sizeof(int2), 0},
+        {pl->batch_unit.data(), pl->batch_unit.size() * sizeof(int), 0},
         {t0.data(), t0.size() * sizeof(double), 0},
         {pl->items.data(), pl->items.size() * sizeof(int2), 0},
         {pl->late.data(), pl->late.size() * sizeof(int2), 0},
@@ -659,8 +646,6 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
         {pl->ref_start.data(), pl->ref_start.size() * sizeof(int), 0},
         {pl->ref_idx.data(), pl->ref_idx.size() * sizeof(int), 0},
         {pl->tile_masks.data(), pl->tile_masks.size() * sizeof(unsigned), 0},
-        {pl->units.data(), pl->units.size() * sizeof(int2), 0},
-        {pl->batch_unit.data(), pl->batch_unit.size() * sizeof(int), 0},
         {r53.data(), r53.size() * sizeof(double), 0},
         {ann_model.data(), ann_model.size() * sizeof(double2), 0},
         {cand.data(), cand.size() * sizeof(double2), 0},
@@ -688,8 +673,8 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.tiles = (const int4*)at(5);
     d.ring_start = (const int*)at(6);
     d.points = (const int2*)at(7);
-    d.wb_start = (const int*)at(8);
-    d.wb_tiles = (const int*)at(9);
+    d.units = (const int2*)at(8);
+    d.batch_unit = (const int*)at(9);
     d.t0 = (const double*)at(10);
     d.items = (const int2*)at(11);
     d.late = (const int2*)at(12);
@@ -702,14 +687,12 @@ extern "C" int sm_plan_create(const sm_channel* ch, int device, sm_plan** out) {
     d.ref_start = (const int*)at(19);
     d.ref_idx = (const int*)at(20);
     d.tile_masks = (const unsigned*)at(21);
-    d.units = (const int2*)at(22);
-    d.batch_unit = (const int*)at(23);
-    d.r53 = (const double*)at(24);
-    d.ann_model = (const double2*)at(25);
-    d.cand = (const double2*)at(26);
-    d.tile_of = (const int*)at(27);
-    d.bis_tasks = (const int4*)at(28);
-    d.bis_lanes = (const int*)at(29);
+    d.r53 = (const double*)at(22);
+    d.ann_model = (const double2*)at(23);
+    d.cand = (const double2*)at(24);
+    d.tile_of = (const int*)at(25);
+    d.bis_tasks = (const int4*)at(26);
+    d.bis_lanes = (const int*)at(27);
     *out = pl;
     return SM_OK;
 }

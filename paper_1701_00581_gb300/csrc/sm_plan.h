@@ -17,7 +17,6 @@ struct sm_plan {
     std::vector<int> bis_lanes;
     std::vector<int> tile_of;        // [w-block][v-block] -> tile id or -1
     int n_vbx = 0, n_vby = 0;
-    std::vector<int> wb_start, wb_tiles;
     std::vector<int> ring_start;
     std::vector<int2> points;
     std::vector<int2> items, units, late;   // phase recursion: early tile rows, units of them, late terms
