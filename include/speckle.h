@@ -202,7 +202,9 @@ int sm_stage_calibrate(const sm_plan* plan, const void* raw, int frame_type, int
  * (sx, sy), |sx|, |sy| <= S, maximising
  * C(s) = sum over the central G x G window of a(x + s) (r(x) - mean r),
  * r the frame `ref` of the burst, the first maximum in row-major (sy, sx)
- * order (products in FP32 over 32-sample chunks, summed in FP64).
+ * order.  Products are summed in FP32 over 32-sample chunks; a thread sums
+ * its chunks as a pair of floats (about 48 bits; in FP64 where such a sum is
+ * not finite), threads and CTAs sum in FP64.
  * ref_window: device float [G][G] scratch; cc: device double
  * [F][2S+1][2S+1] receives C; shifts: device int [F][2] receives (sx, sy).
  * SM_EINVAL unless 0 <= S <= 31 and the window moved by +-S fits the frame
@@ -453,10 +455,7 @@ typedef struct {
                                            inverse and mosaic run on a
                                            high-priority stream beside the
                                            next burst's transforms and
-                                           bispectrum (the recursion takes a
-                                           quarter of an SM and fills the
-                                           issue slots the ALU-bound
-                                           bispectrum leaves);
+                                           bispectrum;
                                            3: batched -- bursts submitted
                                            together (sm_submit_batch) run
                                            through one batched launch
