@@ -223,22 +223,54 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float p) {
     hi = s;
 }
 
-// One shift's products over a thread's share of the window rows [ya, yb) -- of
-// every RB rows those share, share + rs, ... -- from the frame at (x0, y0), as
-// the kernel below forms them, the chunks summed in FP64.
+// A thread's SG shifts over its share of the window rows [ya, yb) -- of every RB
+// rows those share, share + rs, ... -- from column x0 on of the rows at a, the
+// products as the kernel below forms them, the chunks summed in FP64; some
+// shifts at a time, so that the registers of the kernel's own loop suffice, and
+// no further once all of them are NaN.  Columns past the frame, which only
+// shifts past the last one (count) have, are held at its edge.
 template <typename In>
-__device__ __noinline__ double row_share_fp64(const In* a, int W, int x0, int y0, int G, int ya, int yb, int share, int rs,
-                                              const float* rw) {
-    double t = 0.0;
-    for (int yt = ya; yt < yb; yt += RB)
-        for (int y = yt + share; y < min(yt + RB, yb); y += rs)
-            for (int c = 0; c < G; c += 32) {
-                float part = 0.f;
-                for (int x = c; x < min(c + 32, G); ++x)
-                    part = fmaf(sample(a, (size_t)(y0 + y) * W + x0 + x), rw[y * G + x], part);
-                t += (double)part;
+__device__ __forceinline__ void row_share_fp64(const In* a, int W, int x0, int G, int ya, int yb, int share, int rs,
+                                               const float* rw, int count, double* out) {
+    constexpr int N = 6;
+    static_assert(SG % N == 0, "whole groups of shifts");
+#pragma unroll 1
+    for (int k0 = 0; k0 < count; k0 += N) {
+        bool live = true;
+        double t[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) t[k] = 0.0;
+#pragma unroll 1
+        for (int yt = ya; yt < yb && live; yt += RB)
+#pragma unroll 1
+            for (int y = yt + share; y < min(yt + RB, yb) && live; y += rs) {
+                const In* const row = a + (size_t)y * W;
+                float w[N], part[N];
+#pragma unroll
+                for (int k = 1; k < N; ++k) w[k] = sample(row, min(x0 + k0 + k - 1, W - 1));
+#pragma unroll 1
+                for (int c = 0; c < G && live; c += 32) {
+#pragma unroll
+                    for (int k = 0; k < N; ++k) part[k] = 0.f;
+#pragma unroll 4
+                    for (int x = c; x < min(c + 32, G); ++x) {
+#pragma unroll
+                        for (int k = 0; k < N - 1; ++k) w[k] = w[k + 1];
+                        w[N - 1] = sample(row, min(x0 + k0 + x + N - 1, W - 1));
+                        const float r = rw[y * G + x];
+#pragma unroll
+                        for (int k = 0; k < N; ++k) part[k] = fmaf(w[k], r, part[k]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < N; ++k) t[k] += (double)part[k];
+                    live = false;
+#pragma unroll
+                    for (int k = 0; k < N; ++k) live = live || (k0 + k < count && !isnan(t[k]));
+                }
             }
-    return t;
+#pragma unroll
+        for (int k = 0; k < N; ++k) out[k0 + k] = t[k];
+    }
 }
 
 template <typename In>
@@ -317,21 +349,23 @@ k_track_cc(const In* __restrict__ frames, int W, int H, int x0, int y0, int G, i
     double* const red = reinterpret_cast<double*>(smem);                 // [rs][n][ng * SG]
     double* const mine = red + (size_t)sh.rs * sh.slots * SG;            // [n][n]
     const int cw = sh.ng * SG;
+    bool finite = true;
     if (work) {
         double* const own = red + ((size_t)share * n + syi) * cw + s0;
-        bool finite = true;
 #pragma unroll
         for (int k = 0; k < SG; ++k) {
             own[k] = (double)hi[k] + (double)lo[k];
             finite = finite && (s0 + k >= n || isfinite(hi[k]));
         }
-        // a chunk that is not finite, or a sum past the range of a float: this
-        // thread's chunks once more, summed in FP64
-        if (std::is_same<In, float>::value && !finite)
-            for (int k = 0; k < SG && s0 + k < n; ++k)
-                own[k] = row_share_fp64(a, W, x0 + s0 + k - S, y0 + syi - S, G, ya, yb, share, sh.rs, rw);
     }
-    __syncthreads();
+    // chunks that are not finite, or sums past the range of a float: such a
+    // thread's chunks once more, summed in FP64
+    if (__syncthreads_or(std::is_same<In, float>::value && !finite)) {
+        if (!finite)
+            row_share_fp64(a + (size_t)(y0 + syi - S) * W, W, x0 + s0 - S, G, ya, yb, share, sh.rs, rw,
+                           min(SG, n - s0), red + ((size_t)share * n + syi) * cw + s0);
+        __syncthreads();
+    }
     for (int k = tid; k < n * n; k += nt) {
         const int j = k / n, i = k - j * n;
         double t = 0.0;

@@ -36,3 +36,34 @@ def test_sum_past_float_range(G, S):
                 t = a[f, y0 + j - S:y0 + j - S + G, x0 + i - S:x0 + i - S + G]
                 assert abs(got[f, j, i] - (t * r).sum()) <= 67 * 2.0 ** -24 * (np.abs(t) * (np.abs(r) + 4096)).sum()
     assert sh[1].tolist() == [0, 0]
+
+
+def test_time_of_a_burst_that_overflows():
+    """Frames whose every sum overflows, and frames of NaNs, take the FP64 sums in every thread: the first from memory,
+    two loads for six products, the second no further than a chunk.  Both take less than twelve times the time of a
+    finite burst, which has two staged 16-byte loads for 48 products (one shift a thread at a time took fifty)."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("no CUDA device")
+    from paper_1701_00581_gb300 import Channel, Plan
+    F, side, G, S = 100, 512, 256, 16
+    plan = Plan(Channel(W=side, H=side, N=64, R=4, max_frames=F))
+    rw = torch.empty((G, G), dtype=torch.float32, device="cuda:0")
+    cc = torch.empty((F, 2 * S + 1, 2 * S + 1), dtype=torch.float64, device="cuda:0")
+    sh = torch.empty((F, 2), dtype=torch.int32, device="cuda:0")
+    steps = torch.arange(side, device="cuda:0").remainder(2).float()          # columns of 0 and 1: chunks of 16 r
+    ms = {}
+    for name, scale in (("finite", 1.0), ("overflow", 2.5e18), ("nan", float("nan"))):
+        frames = (scale * steps).expand(F, side, side).contiguous()
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t = []
+        for _ in range(4):
+            a.record()
+            plan.stage_track(frames, F, 0, G, S, rw, cc, sh)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        ms[name] = min(t[1:])
+        assert bool(torch.isnan(cc).all()) if name == "nan" else bool(torch.isfinite(cc).all())
+    print(ms)
+    assert max(ms["overflow"], ms["nan"]) < 12 * ms["finite"], ms
